@@ -6,6 +6,7 @@
 // context stream; nothing here allocates device memory.
 #include "../../include/bbc.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -45,7 +46,7 @@ struct Layout {
   size_t ell_chunk, ell, zneed, tasks, group_ptr, group_task, cptr, citem, ccoef, ccoef_df;
   size_t batches, wptr, wunits, qlist, row_slot, orb_ptr, orb_site;
   size_t tc_base, tc_units, row_map, tc_cptr, tc_terms, tc_coefs, dtuples, dchunk, dell, tables_end;
-  size_t stage, prop, amax, kexp, blk, blk16, blkf, blks, P, G, ct, scale, flag, qerr, fftq, total;
+  size_t stage, prop, amax, kexp, blk, blk16, blkf, blks, P, G, ct, scale, flag, qerr, fftq, ex, exE, total;
 };
 
 Layout layout(const bbc_ctx* c, int slots) {
@@ -78,6 +79,10 @@ Layout layout(const bbc_ctx* c, int slots) {
   L.dtuples = o; o = align256(o + sizeof(uint32_t) * c->db.tuples.size());
   L.dchunk = o; o = align256(o + sizeof(int2) * c->db.ell_chunk.size());
   L.dell = o; o = align256(o + sizeof(uint32_t) * c->db.ell.size());
+  {
+    bbc::ExactArgs a;
+    L.ex = o; o = align256(o + (c->exact ? sizeof(int) * bbc::exact_tables(c->ex, nullptr, &a).size() : 0));
+  }
   L.tables_end = o;
   const size_t V = c->V;
   L.stage = o; o = align256(o + (size_t)slots * 2 * V * 144 * 16);
@@ -86,10 +91,12 @@ Layout layout(const bbc_ctx* c, int slots) {
   L.kexp = o; o = align256(o + (size_t)slots * 2 * sizeof(int));
   L.blk = o; o = align256(o + (size_t)slots * V * p.n_out * cplx_bytes(c->prec));
   L.blk16 = o; o = align256(o + (c->prec == BBC_MIXED_BF16 ? (size_t)slots * V * p.n_out * 4 : 0));
-  const bool split = !c->fused;  // the fused path keeps q-major blocks and no product buffer
-  L.blkf = o; o = align256(o + (split ? (size_t)slots * V * p.n_out * cplx_bytes(c->prec) : 0));
+  // field-major blocks beside the site-major ones only for CUDA-core products;
+  // the fused path keeps no product buffer
+  const bool split = !c->fused;
+  L.blkf = o; o = align256(o + (split && !c->exact ? (size_t)slots * V * p.n_out * cplx_bytes(c->prec) : 0));
   // FP64: re + im of every Fourier-space block value (the FP64 products' sums)
-  L.blks = o; o = align256(o + (c->prec == BBC_FP64 ? (size_t)slots * V * p.n_out * sizeof(double) : 0));
+  L.blks = o; o = align256(o + (c->prec == BBC_FP64 && !c->exact ? (size_t)slots * V * p.n_out * sizeof(double) : 0));
   L.P = o; o = align256(o + (split ? (size_t)p.tasks.size() * 16 * V * cplx_bytes(c->prec) : 0));
   // tensor-core products of one slice: G(q) per pair {q, -q}, complex64
   L.G = o; o = align256(o + (c->tc ? c->qlist.size() * (size_t)c->tcs.nbp * c->tcs.nbp * 8 : 0));
@@ -99,6 +106,7 @@ Layout layout(const bbc_ctx* c, int slots) {
   // queue-driven forward FFT: its sticky timeout word, ticket counter and per-tile counters
   L.qerr = o; o = align256(o + sizeof(int));
   L.fftq = o; o = align256(o + (queue_fft(c) ? sizeof(int) * bbc::fft_queue_ints(c->lat.L, slots, p.n_out) : 0));
+  L.exE = o; o = align256(o + (c->exact ? sizeof(int) * slots * (c->ex.jobs.size() / 2) * V : 0));
   L.total = o;
   return L;
 }
@@ -322,6 +330,14 @@ cudaError_t launch_build(bbc_ctx* c, int n_slots, int sites, int threads) {
                                  c->d_blk, p.n_out, real_kind(c->prec), c->stream, sites, threads);
 }
 
+// The digit-sliced products of one slot into P.
+cudaError_t launch_exact(bbc_ctx* c, int slot) {
+  return bbc::launch_contract_exact(c->d_blk + (size_t)slot * c->V * c->plan.n_out * 16, c->lat.L, c->plan.n_out,
+                                    c->prec == BBC_DF64, c->ex_args,
+                                    c->d_exE + (size_t)slot * c->V * c->ex_args.n_jobs, c->d_qlist,
+                                    (int)c->qlist.size(), c->d_P, c->d_qerr, bbc::kFftSpinLimit, c->stream);
+}
+
 // The tensor-core contraction of one slot: G(q) of every pair {q, -q} on
 // the tensor cores, then the CUDA-core products and the Wick sums.  The
 // pairs are cut into chunks: the tensor-core kernel of chunk k + 1 runs on
@@ -432,6 +448,15 @@ bbc_status bbc_create_components(bbc_ctx** ctx, const bbc_lattice* lat, bbc_prec
       c->dense = false;
     }
     if (!c->dense) c->db = bbc::DenseBuild();
+  }
+  if (fp64_storage(prec)) {
+    try {
+      bbc::make_exact_split(c->plan, &c->ex);
+    } catch (const std::bad_alloc&) {
+      delete c;
+      return fail(nullptr, BBC_ENOMEM, "host allocation failed while scheduling");
+    }
+    c->exact = c->ex.all && bbc::exact_wick_smem(16 * (int)c->plan.tasks.size()) <= bbc::kMaxSmemPerBlock;
   }
   // warp task groups of the pair products: enough warps per 32 q to fill the
   // GPU several times over at L = 16 (V/32 q tiles x groups warps); the
@@ -632,7 +657,9 @@ bbc_status bbc_set_workspace(bbc_ctx* c, void* dev_ptr, size_t bytes, int slices
   c->d_blk = w + L.blk;
   c->d_blk16 = w + L.blk16;
   c->d_blkf = w + L.blkf;
-  c->d_blks = c->prec == BBC_FP64 ? (double*)(w + L.blks) : nullptr;
+  c->d_blks = c->prec == BBC_FP64 && !c->exact ? (double*)(w + L.blks) : nullptr;
+  c->d_ex = (int*)(w + L.ex);
+  c->d_exE = (int*)(w + L.exE);
   c->d_P = w + L.P;
   c->d_ct = w + L.ct;
   c->d_scale = (double*)(w + L.scale);
@@ -668,6 +695,12 @@ bbc_status bbc_set_workspace(bbc_ctx* c, void* dev_ptr, size_t bytes, int slices
     wb[i].nA = c->batches[i].nA;
     for (int j = 0; j < 32; j++) wb[i].task[j] = j < wb[i].n ? c->batches[i].tasks[j] : 0;
   }
+  std::vector<int> ex_tables;
+  if (c->exact) {
+    ex_tables = bbc::exact_tables(c->ex, c->d_ex, &c->ex_args);
+    c->ex_args.tasks = c->d_tasks;
+    c->ex_args.n_items = 16 * (int)p.tasks.size();
+  }
   struct Up { void* dst; const void* src; size_t n; } ups[] = {
       {c->d_ell_chunk, p.ell_chunk.data(), sizeof(int2) * p.ell_chunk.size()},
       {c->d_ell, p.ell.data(), sizeof(uint32_t) * p.ell.size()},
@@ -693,6 +726,7 @@ bbc_status bbc_set_workspace(bbc_ctx* c, void* dev_ptr, size_t bytes, int slices
       {c->d_dtuples, c->db.tuples.data(), sizeof(uint32_t) * c->db.tuples.size()},
       {c->d_dchunk, c->db.ell_chunk.data(), sizeof(int2) * c->db.ell_chunk.size()},
       {c->d_dell, c->db.ell.data(), sizeof(uint32_t) * c->db.ell.size()},
+      {c->d_ex, ex_tables.data(), sizeof(int) * ex_tables.size()},
   };
   cudaError_t e0 = cudaMemsetAsync(c->d_qerr, 0, sizeof(int), c->stream);
   if (e0 != cudaSuccess) return cuda_fail(c, e0, "workspace status word");
@@ -775,16 +809,23 @@ bbc_status bbc_build_blocks(bbc_ctx* c, int n_slots) {
   }
   {
     StageScope scope(c, BBC_STAGE_FFT_FWD);
-    // FP64 and unfused FP32: field-major copy for the lanes-over-q products;
-    // fused FP32: in place, q-major
-    e = c->prec == BBC_DF64 ? bbc::launch_fft_forward_df(c->d_blk, c->d_blkf, c->lat.L, n_slots, p.n_out, c->stream)
+    // CUDA-core FP64 and unfused FP32: field-major copy for the lanes-over-q products;
+    // digit-sliced products and fused FP32: in place, q-major
+    e = c->exact            ? bbc::launch_fft_forward_site(c->d_blk, c->lat.L, n_slots, p.n_out, real_kind(c->prec),
+                                                           c->stream)
+        : c->prec == BBC_DF64 ? bbc::launch_fft_forward_df(c->d_blk, c->d_blkf, c->lat.L, n_slots, p.n_out, c->stream)
         : !c->fused         ? bbc::launch_fft_forward(c->d_blk, c->d_blkf, c->lat.L, n_slots, p.n_out, fp64, c->stream,
                                                       c->d_blks)
         : queue_fft(c)      ? bbc::launch_fft_forward_queue(c->d_blk, c->lat.L, n_slots, p.n_out,
                                                         bbc::FftQueue{c->d_fftq, c->d_qerr}, -1, bbc::kFftSpinLimit,
                                                         c->stream)
-                            : bbc::launch_fft_forward_site(c->d_blk, c->lat.L, n_slots, p.n_out, fp64, c->stream);
+                            : bbc::launch_fft_forward_site(c->d_blk, c->lat.L, n_slots, p.n_out, bbc::RK_F32, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "forward FFT");
+    if (c->exact) {
+      e = bbc::launch_exact_exponents(c->d_blk, c->prec == BBC_DF64, (long long)n_slots * c->V, p.n_out,
+                                      c->ex_args.jobs, c->ex_args.n_jobs, c->d_exE, c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "row exponents");
+    }
     if (c->prec == BBC_MIXED_BF16) {
       e = bbc::launch_to_bf16(c->d_blk, c->d_blk16, (size_t)n_slots * c->V * p.n_out, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "bfloat16 rounding");
@@ -803,13 +844,25 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
   const bool fp64 = fp64_storage(c->prec);
   const bbc::Plan& p = c->plan;
   const int n_ch = (int)p.channels.size();
+  bbc::ScaleParams sp{};
+  sp.n_ch = n_ch;
+  const int t = c->slot_t[slot];
+  const int d = time_distance(c, t);
+  for (int i = 0; i < n_ch; i++) {
+    const int ns = p.n_strange[i];
+    const double mass = (6 - ns) * c->lat.m_ud + ns * c->lat.m_s;  // m_B1 + m_B2
+    sp.f[i] = (1.0 / c->V) * (normalised ? std::exp(mass * d) : 1.0);
+    sp.nl[i] = 6 - ns;
+    sp.ns[i] = ns;
+  }
   cudaError_t e;
   if (!c->fused) {
     const char* blkf = c->d_blkf + (size_t)slot * c->V * p.n_out * cplx_bytes(c->prec);
     const double* blks = c->d_blks ? c->d_blks + (size_t)slot * c->V * p.n_out : nullptr;
     {
       StageScope scope(c, BBC_STAGE_CONTRACT);
-      e = c->prec == BBC_DF64
+      e = c->exact ? launch_exact(c, slot)
+          : c->prec == BBC_DF64
               ? bbc::launch_pair_products_df(blkf, c->lat.L, c->d_tasks, c->d_group_ptr, c->d_group_task,
                                              (int)c->group_ptr.size() - 1, c->d_P, c->stream)
               : bbc::launch_pair_products(blkf, c->lat.L, c->d_tasks, c->d_group_ptr, c->d_group_task,
@@ -818,7 +871,9 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
     }
     {
       StageScope scope(c, BBC_STAGE_WICK);
-      e = c->prec == BBC_DF64
+      e = c->exact ? bbc::launch_exact_wick(c->d_P, c->V, c->ex_args.n_items, c->d_cptr, c->d_citem, c->d_ccoef,
+                                            c->d_ccoef_df, n_ch * 16, c->d_ct, c->prec == BBC_DF64, c->stream)
+          : c->prec == BBC_DF64
               ? bbc::launch_wick_sums_df(c->d_P, c->lat.L, c->d_cptr, c->d_citem, c->d_ccoef_df, n_ch, c->d_ct,
                                          c->stream)
               : bbc::launch_wick_sums(c->d_P, c->lat.L, c->d_cptr, c->d_citem, c->d_ccoef, n_ch, c->d_ct, fp64,
@@ -841,17 +896,6 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
                                    c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "fused contraction");
   }
-  bbc::ScaleParams sp{};
-  sp.n_ch = n_ch;
-  const int t = c->slot_t[slot];
-  const int d = time_distance(c, t);
-  for (int i = 0; i < n_ch; i++) {
-    const int ns = p.n_strange[i];
-    const double mass = (6 - ns) * c->lat.m_ud + ns * c->lat.m_s;  // m_B1 + m_B2
-    sp.f[i] = (1.0 / c->V) * (normalised ? std::exp(mass * d) : 1.0);
-    sp.nl[i] = 6 - ns;
-    sp.ns[i] = ns;
-  }
   {
     StageScope scope(c, BBC_STAGE_NORMALISE);
     e = bbc::launch_scales(sp, c->d_kexp + slot * 2, c->d_scale, c->stream);
@@ -859,7 +903,10 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
   }
   {
     StageScope scope(c, BBC_STAGE_FFT_INV);
-    e = c->prec == BBC_DF64 ? bbc::launch_fft_inverse_df(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, c->stream)
+    e = c->exact && c->prec == BBC_DF64
+            ? bbc::launch_fft_inverse_site_df(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, c->stream)
+        : c->exact ? bbc::launch_fft_inverse_site(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, true, c->stream)
+        : c->prec == BBC_DF64 ? bbc::launch_fft_inverse_df(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, c->stream)
         : !c->fused ? bbc::launch_fft_inverse(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, fp64, c->stream)
                : bbc::launch_fft_inverse_site(c->d_ct, out_dev, c->lat.L, n_ch, c->d_scale, fp64, c->stream, c->tc);
     if (e != cudaSuccess) return cuda_fail(c, e, "inverse FFT");
@@ -1051,6 +1098,11 @@ bbc_status bbc_autotune(bbc_ctx* c, int reps, bbc_tuning* best, double* ms, int 
       }
       c->tune.tc_kernel = t.tc_kernel;
     }
+  } else if (c->exact) {
+    // the digit-sliced products have no task lists: one timing stands for every pair_groups value
+    const double v = time_launches(c, reps, [&] { return launch_exact(c, 0); });
+    if (v < 0) return cuda_fail(c, cudaGetLastError(), "autotune: digit-sliced products");
+    for (size_t i = 0; i < sizeof(kPairGroupsCand) / sizeof(kPairGroupsCand[0]); i++) record(v);
   } else {  // block-pair products: task lists per 32 q
     const bool fp64 = fp64_storage(c->prec);
     const double* blks = c->d_blks;
@@ -1226,16 +1278,17 @@ bbc_status bbc_stage_timing(bbc_ctx* c, double* ms, long long* launches) {
 
 bbc_status bbc_launch_counts(const bbc_ctx* c, int* per_load, int* per_build, int* per_contract) {
   if (!c) return BBC_EINVAL;
-  // forward and inverse FFT passes: the fused (q-major) layout fuses the x and
-  // y passes for L <= 32 (and runs the forward transform as one queue-driven
-  // launch there); the field-major layout runs three
-  const bool xy = c->fused && c->lat.L <= 32;
-  const int passes = xy ? 2 : 3;
+  // forward and inverse FFT passes: the q-major layout fuses the x and y passes
+  // for L <= 32 (and the fused FP32 path runs the forward transform as one
+  // queue-driven launch there); the field-major layout runs three
+  const int passes = c->fused || c->exact ? bbc::fft_site_passes(c->lat.L) : 3;
   const int fwd = queue_fft(c) ? 1 : passes;
   if (per_load) *per_load = 2;  // absmax, convert
-  if (per_build) *per_build = 1 + fwd + (c->prec == BBC_MIXED_BF16 ? 1 : 0);  // build, FFT (, bfloat16 rounding)
-  // contraction kernel(s), scales, inverse passes
-  if (per_contract) *per_contract = (c->tc ? 2 : c->fused ? 1 : 2) + 1 + passes;
+  // build, FFT (, row exponents or bfloat16 rounding)
+  if (per_build) *per_build = 1 + fwd + (c->exact || c->prec == BBC_MIXED_BF16 ? 1 : 0);
+  // contraction kernel(s), Wick sums, scales, inverse passes
+  const int products = c->exact ? 1 + !c->ex.small.empty() : c->tc ? 2 : 1;
+  if (per_contract) *per_contract = products + (c->fused ? 0 : 1) + 1 + passes;
   return BBC_OK;
 }
 

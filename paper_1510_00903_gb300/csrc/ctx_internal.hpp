@@ -1,6 +1,7 @@
 // ctx_internal.hpp -- definition of the opaque bbc_ctx (internal to libbbc).
 #pragma once
 
+#include <cstring>
 #include <string>
 #include <utility>
 #include <vector>
@@ -32,8 +33,15 @@ struct bbc_ctx {
   int* d_citem = nullptr;
   double* d_ccoef = nullptr;
   float2* d_ccoef_df = nullptr;          // the coefficients as double-float pairs (BBC_DF64)
-  std::vector<int> group_ptr;            // warp task groups of the pair products (FP64)
+  std::vector<int> group_ptr;            // warp task groups of the pair products on the CUDA cores
   std::vector<int> group_task;
+  // FP64 / double-float with digit-sliced tensor-core products (q-major blocks,
+  // transformed in place); else field-major blocks and CUDA-core products
+  bbc::ExactSplit ex;
+  bool exact = false;
+  int* d_ex = nullptr;                   // the sets' tables (exact_tables)
+  bbc::ExactArgs ex_args = {};           // device pointers into them
+  int* d_exE = nullptr;                  // [slots][V][jobs] row exponents
   // fused FP32 contraction: warp batches, per-warp units, one q per pair {q, -q}
   std::vector<bbc::Batch> batches;
   std::vector<int> wptr;
@@ -137,6 +145,48 @@ inline void to_dev_tasks(const PairTask* src, size_t n, const std::vector<int>* 
     d.sA = t.sA1 | (t.sA2 << 16);
     d.sB = t.sB1 | (t.sB2 << 16);
   }
+}
+
+// Device tables of the digit-sliced sets, packed into one array of ints: jobs
+// and small tasks, then per set rowA, rowB, expA, expB and the needed entries (padded to 16
+// bytes); *a points into it at `base`.
+inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, ExactArgs* a) {
+  std::vector<int> t;
+  auto put = [&](const void* src, size_t bytes) {
+    const size_t at = t.size();
+    t.resize(at + (bytes + 15) / 16 * 4, 0);
+    if (bytes) std::memcpy(t.data() + at, src, bytes);
+    return base + at;
+  };
+  a->n_jobs = (int)s.jobs.size() / 2;
+  a->n_small = (int)s.small.size();
+  a->jobs = put(s.jobs.data(), sizeof(int) * s.jobs.size());
+  a->small = put(s.small.data(), sizeof(int) * s.small.size());
+  const ExactSet* sets[2] = {&s.trace, &s.slice};
+  for (int i = 0; i < 2; i++) {
+    const ExactSet& x = *sets[i];
+    ExactDev& d = i == 0 ? a->trace : a->slice;
+    d.nA = (int)x.rowA.size();
+    d.nB = (int)x.rowB.size();
+    d.nAp = x.nAp;
+    d.nBp = x.nBp;
+    d.K = i == 0 ? 144 : 36;
+    d.rowA = put(x.rowA.data(), sizeof(int) * x.rowA.size());
+    d.rowB = put(x.rowB.data(), sizeof(int) * x.rowB.size());
+    d.expA = put(x.expA.data(), sizeof(int) * x.expA.size());
+    d.expB = put(x.expB.data(), sizeof(int) * x.expB.size());
+    std::vector<int> ent;
+    for (int c = 0; c < x.nBp; c++)
+      for (int r = 0; r < x.nAp; r++) {
+        const short iq = x.itemQ[(size_t)r * x.nBp + c], in = x.itemNQ[(size_t)r * x.nBp + c];
+        if (iq < 0 && in < 0) continue;
+        ent.push_back(r | (c << 16));
+        ent.push_back((int)((unsigned)(unsigned short)iq | ((unsigned)(unsigned short)in << 16)));
+      }
+    d.n_ent = (int)ent.size() / 2;
+    d.entries = (const int2*)put(ent.data(), sizeof(int) * ent.size());
+  }
+  return t;
 }
 
 static_assert(N_DIQUARK == kMaxDiquarks && N_FAMILY == kMaxFamilies && kMaxGroups == kMaxBuildGroups,

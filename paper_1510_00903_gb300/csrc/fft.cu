@@ -189,28 +189,27 @@ enum { FFT_SITE2FIELD = 0, FFT_FIELD = 1, FFT_FIELD2OUT = 2, FFT_SITE = 3, FFT_S
 // compute type, O: storage of the output of the last inverse pass.
 template <typename S, typename R, int N, bool INV, int MODE, typename O = S>
 __global__ void __launch_bounds__(256)
-k_fft(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n_outer, int n_inner, int axis,
+k_fft(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned total, int n_inner, int axis,
       const double* __restrict__ scale, O* __restrict__ sum) {
-  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int lines = N * N;
+  // 32-bit indices (fft_dispatch cuts larger launches)
+  const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned lines = N * N;
   const long long V = (long long)N * N * N;
+  if (gid >= total) return;
   int line, inner;
   long long o;
   if (MODE == FFT_SITE2FIELD || MODE == FFT_SITE || MODE == FFT_SITE2OUT) {
-    if (gid >= n_outer * lines * n_inner) return;
-    inner = (int)(gid % n_inner);
-    const long long rest = gid / n_inner;
+    inner = (int)(gid % (unsigned)n_inner);
+    const unsigned rest = gid / (unsigned)n_inner;
     line = (int)(rest % lines);
     o = rest / lines;
   } else if (MODE == FFT_FIELD || MODE == FFT_FIELD_SUM) {
-    if (gid >= n_outer * lines) return;
     line = (int)(gid % lines);
     o = gid / lines;
     inner = 0;
   } else {  // FIELD2OUT: spin fastest so that each site's 16 spins are written together
-    if (gid >= n_outer * lines * 16) return;
     inner = (int)(gid % 16);
-    const long long rest = gid / 16;
+    const unsigned rest = gid / 16;
     line = (int)(rest % lines);
     o = rest / lines;  // channel
   }
@@ -269,12 +268,11 @@ k_fft(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n_outer
 // applies the twiddles exp(-+2 pi i j k2 / N) and leaves the result in shared
 // memory; after a barrier, thread j combines k2 = j, j + 3, ... with the
 // radix-3 butterfly into X[k2], X[k2 + M], X[k2 + 2M] and stores them.  The
-// modes, index decomposition and output forms are those of k_fft
-// (FIELD-type passes and the site-major first pass).
+// modes, index decomposition and output forms are those of k_fft.
 constexpr int kSplitLines = 64;  // lines per CTA of 3 x 64 threads
 template <typename S, typename R, int M, bool INV, int MODE, typename O = S>
 __global__ void __launch_bounds__(3 * kSplitLines)
-k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n_outer, int n_inner, int axis,
+k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned total, int n_inner, int axis,
             const double* __restrict__ scale, O* __restrict__ sum) {
   constexpr int N = 3 * M;
   // sh[line][j][k2 ^ (line & 7)]: a line's 3 M values are 3 M x 16 bytes
@@ -285,26 +283,23 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
   __shared__ cpx<R> sh[kSplitLines][3][M];
   auto at = [&](int l, int jj, int k2) -> cpx<R>& { return sh[l][jj][k2 ^ (l & 7)]; };
   const int ls = threadIdx.x % kSplitLines, j = threadIdx.x / kSplitLines;
-  const long long gid = blockIdx.x * (long long)kSplitLines + ls;
-  const int lines = N * N;
+  const unsigned gid = blockIdx.x * kSplitLines + ls;
+  const unsigned lines = N * N;
   const long long V = (long long)N * N * N;
   int line = 0, inner = 0;
   long long o = 0;
-  bool live;
-  if (MODE == FFT_SITE2FIELD) {
-    live = gid < n_outer * lines * n_inner;
-    inner = (int)(gid % n_inner);
-    const long long rest = gid / n_inner;
+  const bool live = gid < total;
+  if (MODE == FFT_SITE2FIELD || MODE == FFT_SITE || MODE == FFT_SITE2OUT) {
+    inner = (int)(gid % (unsigned)n_inner);
+    const unsigned rest = gid / (unsigned)n_inner;
     line = (int)(rest % lines);
     o = rest / lines;
   } else if (MODE == FFT_FIELD || MODE == FFT_FIELD_SUM) {
-    live = gid < n_outer * lines;
     line = (int)(gid % lines);
     o = gid / lines;
   } else {  // FIELD2OUT
-    live = gid < n_outer * lines * 16;
     inner = (int)(gid % 16);
-    const long long rest = gid / 16;
+    const unsigned rest = gid / 16;
     line = (int)(rest % lines);
     o = rest / lines;
   }
@@ -313,7 +308,7 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
   if (live) {
     const cpx<S>* p;
     long long step;
-    if (MODE == FFT_SITE2FIELD) { p = in + (o * V + base) * n_inner + inner; step = (long long)stride * n_inner; }
+    if (MODE == FFT_SITE2FIELD || MODE == FFT_SITE || MODE == FFT_SITE2OUT) { p = in + (o * V + base) * n_inner + inner; step = (long long)stride * n_inner; }
     else if (MODE == FFT_FIELD || MODE == FFT_FIELD_SUM) { p = in + o * V + base; step = stride; }
     else { p = in + (o * 16 + inner) * V + base; step = stride; }
     cpx<R> u[M];
@@ -356,12 +351,11 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
     // the next by additions, not recomputed with 64-bit divisions per point
     constexpr int kStep = 3 * kSplitLines / N;
     static_assert(kStep * N == 3 * kSplitLines, "whole lines per round of stores");
-    const long long total = n_outer * lines * n_inner;
     const int k = threadIdx.x % N, kj = k / M, kk = k % M;
     int l = threadIdx.x / N;
-    long long gl = blockIdx.x * (long long)kSplitLines + l;
-    int inn = (int)(gl % n_inner), ln = (int)((gl / n_inner) % lines);
-    long long oo = gl / n_inner / lines;
+    unsigned gl = blockIdx.x * kSplitLines + l;
+    int inn = (int)(gl % (unsigned)n_inner), ln = (int)((gl / (unsigned)n_inner) % lines);
+    long long oo = gl / (unsigned)n_inner / lines;
     for (; l < kSplitLines && gl < total; l += kStep) {  // lines past the end come last
       int b = 0, sd = 0;
       line_base(N, axis, ln, b, sd);
@@ -370,7 +364,7 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
       inn += kStep;
       while (inn >= n_inner) {
         inn -= n_inner;
-        if (++ln == lines) {
+        if (++ln == (int)lines) {
           ln = 0;
           ++oo;
         }
@@ -390,6 +384,12 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
       const int k = k2 + c * M;
       if (MODE == FFT_FIELD) {
         out[o * V + base + (long long)k * stride] = cpx<O>(x[c]);
+      } else if (MODE == FFT_SITE) {
+        out[(o * V + base + (long long)k * stride) * n_inner + inner] = cpx<O>(x[c]);
+      } else if (MODE == FFT_SITE2OUT) {  // inner = channel * 16 + spin
+        const O f = (O)scale[inner >> 4];
+        out[((long long)(inner >> 4) * V + base + (long long)k * stride) * 16 + (inner & 15)] =
+            cpx<O>((O)x[c].re * f, (O)x[c].im * f);
       } else if (MODE == FFT_FIELD_SUM) {
         const cpx<O> w(x[c]);
         out[o * V + base + (long long)k * stride] = w;
@@ -407,14 +407,14 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, long long n
 // columns, stages the N x N x TI plane in shared memory (compute precision),
 // runs the x lines there, then the y lines, writing the result in place.
 // One HBM round trip for two passes.
-template <int N>
-__host__ __device__ constexpr int xy_tile() {
-  return N <= 16 ? 32 : (N == 24 ? 16 : (N == 32 ? 8 : 4));  // planes of <= 74 KB
+template <int N, typename R>
+__host__ __device__ constexpr int xy_tile() {  // planes of <= 74 KB
+  return N <= 8 ? 32 : N == 16 ? (sizeof(R) == 8 ? 16 : 32) : N == 24 ? 16 : 8;
 }
 
 template <typename S, typename R, int N, bool INV>
 __global__ void __launch_bounds__(256) k_fft_xy_site(cpx<S>* __restrict__ data, int n_inner) {
-  constexpr int TI = xy_tile<N>();
+  constexpr int TI = xy_tile<N, R>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* tile = reinterpret_cast<cpx<R>*>(smem_raw);  // [N * N][TI]
   const int i0 = blockIdx.x * TI, z = blockIdx.y;
@@ -446,33 +446,161 @@ __global__ void __launch_bounds__(256) k_fft_xy_site(cpx<S>* __restrict__ data, 
   }
 }
 
-template <typename S, typename R>
-static cudaError_t fft_xy_site(void* data, int L, long long n_outer, int n_inner, bool inv, cudaStream_t st) {
-#define BBC_XY_CASE(NN)                                                                                          \
-  case NN: {                                                                                                     \
-    constexpr int TI = xy_tile<NN>();                                                                            \
-    const size_t sm = sizeof(cpx<R>) * NN * NN * TI;                                                             \
-    dim3 grid((unsigned)((n_inner + TI - 1) / TI), NN, (unsigned)n_outer);                                      \
-    static int granted_f[64] = {0}, granted_i[64] = {0};                                                         \
-    cudaError_t e = inv ? ensure_smem(k_fft_xy_site<S, R, NN, true>, sm, granted_i)                              \
-                        : ensure_smem(k_fft_xy_site<S, R, NN, false>, sm, granted_f);                            \
-    if (e != cudaSuccess) return e;                                                                              \
-    if (inv) k_fft_xy_site<S, R, NN, true><<<grid, 256, sm, st>>>((cpx<S>*)data, n_inner);                       \
-    else k_fft_xy_site<S, R, NN, false><<<grid, 256, sm, st>>>((cpx<S>*)data, n_inner);                          \
-    break;                                                                                                       \
+// The same fusion with every line split over SPLIT threads (N = SPLIT M, M a
+// power of two): thread j of a line transforms x[SPLIT n2 + j] (M values in
+// registers), applies the twiddles and puts u_j[k2] at position j M + k2 of the
+// line; thread j then joins k2 = j, j + SPLIT, ... with a radix-SPLIT butterfly
+// whose inputs and outputs share their positions.  For 16-byte values a whole
+// line of 24 or more points in one thread leaves one CTA per SM; the split lines
+// keep two or more, so one CTA's loads overlap another's arithmetic (double-float
+// forward transform of a 24^3 slice: 1.9 ms, with whole lines 3.6, field-major
+// 2.9).  Bound by FP32 issue (double-float) or the FP64 pipe.  At 48 points a
+// plane leaves room for tiles of 2 or 4 columns only: 10.9 and 13.1 ms per
+// 48^3 slice for the two passes against 10.1 as two launches, so it keeps those.
+// A plane row (fixed y) is padded by one tile row so that the x lines of
+// neighbouring y fall in different banks.
+template <int N>
+struct XySplit {};
+template <>
+struct XySplit<24> { static constexpr int kSplit = 3, kTile = 8, kCtas = 2; };
+template <>
+struct XySplit<32> { static constexpr int kSplit = 2, kTile = 4, kCtas = 2; };
+
+// position of (x, y, i) in the staged plane
+template <int N, int TI>
+__device__ __forceinline__ int xy_pos(int x, int y, int i) { return (y * N + x) * TI + i + (TI < 8 ? y * TI : 0); }
+template <int N, int TI>
+__host__ __device__ constexpr int xy_elems() { return N * N * TI + (TI < 8 ? N * TI : 0); }
+
+template <typename R, int N, int SPLIT, bool INV, typename Pos>
+__device__ __forceinline__ void xy_split_first(cpx<R>* tile, int j, cpx<R> (&v)[N / SPLIT], Pos pos) {
+  constexpr int M = N / SPLIT;
+#pragma unroll
+  for (int k = 0; k < M; k++) v[bitrev(k, M)] = tile[pos(SPLIT * k + j)];
+  fft_pow2<R, M, INV>(v);
+#pragma unroll
+  for (int k2 = 0; k2 < M; k2++) {
+    const int ti = (j * k2 * (kTw / N)) % kTw;
+    if (ti != 0) {
+      cpx<R> w = twiddle<R>(ti);
+      if (INV) w.im = -w.im;
+      v[k2] = w * v[k2];
+    }
   }
+}
+// radix-SPLIT butterfly of the (twiddled) values of one k2: X[k2 + c M] = out[c]
+template <typename R, int SPLIT, bool INV>
+__device__ __forceinline__ void xy_join(const cpx<R> (&t)[SPLIT], cpx<R> (&x)[SPLIT]) {
+  if constexpr (SPLIT == 2) {
+    x[0] = t[0] + t[1];
+    x[1] = t[0] - t[1];
+  } else {
+    const R hs = (R)0.86602540378443864676;  // sqrt(3)/2
+    const cpx<R> sm = t[1] + t[2], d = t[1] - t[2];
+    const cpx<R> m(t[0].re - (R)0.5 * sm.re, t[0].im - (R)0.5 * sm.im);
+    const cpx<R> r = INV ? cpx<R>(-hs * d.im, hs * d.re) : cpx<R>(hs * d.im, -hs * d.re);
+    x[0] = t[0] + sm;
+    x[1] = m + r;
+    x[2] = m - r;
+  }
+}
+
+template <typename R, int N, bool INV>
+__global__ void __launch_bounds__(N * XySplit<N>::kTile * XySplit<N>::kSplit, XySplit<N>::kCtas)
+k_fft_xy_split(cpx<R>* __restrict__ data, int n_inner) {
+  constexpr int TI = XySplit<N>::kTile, SPLIT = XySplit<N>::kSplit, M = N / SPLIT, T = N * TI * SPLIT;
+  static_assert(sizeof(cpx<R>) == 16, "16-byte asynchronous copies");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpx<R>* tile = reinterpret_cast<cpx<R>*>(smem_raw);
+  const int i0 = blockIdx.x * TI, z = blockIdx.y, tid = threadIdx.x;
+  cpx<R>* plane = data + ((long long)blockIdx.z * N * N * N + (long long)z * N * N) * n_inner + i0;
+  const int i = tid % TI, a = tid / TI % N, j = tid / (TI * N);  // line (a, i), thread j of it
+  const bool in = i0 + i < n_inner;
+  // rows of TI values of one site; T / TI sites per round
+  for (int site = tid / TI; site < N * N; site += T / TI) {
+    cpx<R>* dst = tile + xy_pos<N, TI>(site % N, site / N, i);
+    if (in) cp_async16(dst, plane + (long long)site * n_inner + i);
+    else *dst = cpx<R>((R)0, (R)0);
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  cpx<R> v[M], t[SPLIT], x[SPLIT];
+  {
+    auto pos = [&](int k) { return xy_pos<N, TI>(k, a, i); };  // x lines: (y = a, i)
+    xy_split_first<R, N, SPLIT, INV>(tile, j, v, pos);
+    __syncthreads();
+#pragma unroll
+    for (int k2 = 0; k2 < M; k2++) tile[pos(j * M + k2)] = v[k2];
+    __syncthreads();
+    for (int k2 = j; k2 < M; k2 += SPLIT) {
+#pragma unroll
+      for (int c = 0; c < SPLIT; c++) t[c] = tile[pos(c * M + k2)];
+      xy_join<R, SPLIT, INV>(t, x);
+#pragma unroll
+      for (int c = 0; c < SPLIT; c++) tile[pos(c * M + k2)] = x[c];
+    }
+    __syncthreads();
+  }
+  {
+    auto pos = [&](int k) { return xy_pos<N, TI>(a, k, i); };  // y lines: (x = a, i), to global memory
+    xy_split_first<R, N, SPLIT, INV>(tile, j, v, pos);
+    __syncthreads();
+#pragma unroll
+    for (int k2 = 0; k2 < M; k2++) tile[pos(j * M + k2)] = v[k2];
+    __syncthreads();
+    for (int k2 = j; k2 < M; k2 += SPLIT) {
+#pragma unroll
+      for (int c = 0; c < SPLIT; c++) t[c] = tile[pos(c * M + k2)];
+      xy_join<R, SPLIT, INV>(t, x);
+      if (in) {
+#pragma unroll
+        for (int c = 0; c < SPLIT; c++) plane[(long long)(a + N * (c * M + k2)) * n_inner + i] = x[c];
+      }
+    }
+  }
+}
+
+template <typename R, int N, bool INV>
+static cudaError_t launch_xy_split(void* data, long long n_outer, int n_inner, cudaStream_t st) {
+  constexpr int TI = XySplit<N>::kTile, T = N * TI * XySplit<N>::kSplit;
+  constexpr size_t sm = sizeof(cpx<R>) * xy_elems<N, TI>();
+  static int granted[64] = {0};
+  cudaError_t e = ensure_smem(k_fft_xy_split<R, N, INV>, sm, granted);
+  if (e != cudaSuccess) return e;
+  k_fft_xy_split<R, N, INV><<<dim3((unsigned)((n_inner + TI - 1) / TI), N, (unsigned)n_outer), T, sm, st>>>(
+      (cpx<R>*)data, n_inner);
+  return cudaGetLastError();
+}
+
+template <typename S, typename R, int N, bool INV>
+static cudaError_t launch_xy_site(void* data, long long n_outer, int n_inner, cudaStream_t st) {
+  constexpr int TI = xy_tile<N, R>();
+  constexpr size_t sm = sizeof(cpx<R>) * N * N * TI;
+  static int granted[64] = {0};
+  cudaError_t e = ensure_smem(k_fft_xy_site<S, R, N, INV>, sm, granted);
+  if (e != cudaSuccess) return e;
+  k_fft_xy_site<S, R, N, INV><<<dim3((unsigned)((n_inner + TI - 1) / TI), N, (unsigned)n_outer), 256, sm, st>>>(
+      (cpx<S>*)data, n_inner);
+  return cudaGetLastError();
+}
+
+template <typename S, typename R, bool INV>
+static cudaError_t fft_xy_site(void* data, int L, long long n_outer, int n_inner, cudaStream_t st) {
+  // 16-byte values: split lines from 24 points
+  constexpr bool wide = sizeof(R) == 8 && std::is_same<S, R>::value;
   switch (L) {
-    BBC_XY_CASE(2)
-    BBC_XY_CASE(4)
-    BBC_XY_CASE(8)
-    BBC_XY_CASE(16)
-    BBC_XY_CASE(24)
-    BBC_XY_CASE(32)
-    BBC_XY_CASE(48)
+    case 2: return launch_xy_site<S, R, 2, INV>(data, n_outer, n_inner, st);
+    case 4: return launch_xy_site<S, R, 4, INV>(data, n_outer, n_inner, st);
+    case 8: return launch_xy_site<S, R, 8, INV>(data, n_outer, n_inner, st);
+    case 16: return launch_xy_site<S, R, 16, INV>(data, n_outer, n_inner, st);
+    case 24:
+      if constexpr (wide) return launch_xy_split<R, 24, INV>(data, n_outer, n_inner, st);
+      else return launch_xy_site<S, R, 24, INV>(data, n_outer, n_inner, st);
+    case 32:
+      if constexpr (wide) return launch_xy_split<R, 32, INV>(data, n_outer, n_inner, st);
+      else return launch_xy_site<S, R, 32, INV>(data, n_outer, n_inner, st);
     default: return cudaErrorInvalidValue;
   }
-#undef BBC_XY_CASE
-  return cudaGetLastError();
 }
 
 // ------------------------------------------------ persistent site-major FFT
@@ -718,23 +846,35 @@ static cudaError_t fft_dispatch(const void* in, void* out, int L, long long n_ou
                                 const double* scale, cudaStream_t st, O* sum = nullptr) {
   long long per = (MODE == FFT_SITE2FIELD || MODE == FFT_SITE || MODE == FFT_SITE2OUT) ? n_inner
                   : ((MODE == FFT_FIELD || MODE == FFT_FIELD_SUM) ? 1 : 16);
-  long long total = n_outer * (long long)L * L * per;
-  unsigned blocks = (unsigned)((total + 255) / 256);
+  const long long total = n_outer * (long long)L * L * per;
   const cpx<S>* i = (const cpx<S>*)in;
   cpx<O>* o = (cpx<O>*)out;
-  if constexpr (sizeof(R) == 8 && MODE != FFT_SITE && MODE != FFT_SITE2OUT) {
+  if (total >= (1ll << 31)) {  // the kernels index with 32 bits: halves of the outer index
+    if constexpr (MODE == FFT_SITE2OUT) {
+      return cudaErrorInvalidValue;  // one outer index
+    } else {
+      if (n_outer < 2) return cudaErrorInvalidValue;
+      const long long h = n_outer / 2, in_step = h * L * L * L * per, out_step = in_step;
+      cudaError_t e = fft_dispatch<S, R, MODE, O>(i, o, L, h, n_inner, axis, inv, scale, st, sum);
+      if (e != cudaSuccess) return e;
+      return fft_dispatch<S, R, MODE, O>(i + in_step, o + out_step, L, n_outer - h, n_inner, axis, inv,
+                                         scale ? scale + h : nullptr, st, sum ? sum + out_step : nullptr);
+    }
+  }
+  const unsigned blocks = (unsigned)((total + 255) / 256);
+  if constexpr (sizeof(R) == 8) {
     // FP64 and double-float 48-point lines: three threads per line
     if (L == 48) {
       const unsigned b3 = (unsigned)((total + kSplitLines - 1) / kSplitLines);
-      if (inv) k_fft3split<S, R, 16, true, MODE, O><<<b3, 3 * kSplitLines, 0, st>>>(i, o, n_outer, n_inner, axis, scale, sum);
-      else k_fft3split<S, R, 16, false, MODE, O><<<b3, 3 * kSplitLines, 0, st>>>(i, o, n_outer, n_inner, axis, scale, sum);
+      if (inv) k_fft3split<S, R, 16, true, MODE, O><<<b3, 3 * kSplitLines, 0, st>>>(i, o, (unsigned)total, n_inner, axis, scale, sum);
+      else k_fft3split<S, R, 16, false, MODE, O><<<b3, 3 * kSplitLines, 0, st>>>(i, o, (unsigned)total, n_inner, axis, scale, sum);
       return cudaGetLastError();
     }
   }
 #define BBC_FFT_CASE(NN)                                                                                      \
   case NN:                                                                                                    \
-    if (inv) k_fft<S, R, NN, true, MODE, O><<<blocks, 256, 0, st>>>(i, o, n_outer, n_inner, axis, scale, sum); \
-    else k_fft<S, R, NN, false, MODE, O><<<blocks, 256, 0, st>>>(i, o, n_outer, n_inner, axis, scale, sum);     \
+    if (inv) k_fft<S, R, NN, true, MODE, O><<<blocks, 256, 0, st>>>(i, o, (unsigned)total, n_inner, axis, scale, sum); \
+    else k_fft<S, R, NN, false, MODE, O><<<blocks, 256, 0, st>>>(i, o, (unsigned)total, n_inner, axis, scale, sum);     \
     break;
   switch (L) {
     BBC_FFT_CASE(2)
@@ -790,21 +930,33 @@ cudaError_t launch_fft_forward_df(const void* blk_site, void* blk_field, int L, 
   return cudaSuccess;
 }
 
-cudaError_t launch_fft_forward_site(void* blk, int L, int n_slots, int n_rows, bool fp64, cudaStream_t st) {
-  cudaError_t e;
-  if (L <= 32) {  // x and y fused (one HBM round trip), then z
-    e = fp64 ? fft_xy_site<double, double>(blk, L, n_slots, n_rows, false, st)
-             : fft_xy_site<float, float>(blk, L, n_slots, n_rows, false, st);
-    if (e != cudaSuccess) return e;
-  } else {  // L = 48: the 48-point lines leave too few registers for a fused plane
-    for (int axis = 0; axis < 2; axis++) {
-      e = fp64 ? fft_dispatch<double, double, FFT_SITE>(blk, blk, L, n_slots, n_rows, axis, false, nullptr, st)
-               : fft_dispatch<float, float, FFT_SITE>(blk, blk, L, n_slots, n_rows, axis, false, nullptr, st);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return fp64 ? fft_dispatch<double, double, FFT_SITE>(blk, blk, L, n_slots, n_rows, 2, false, nullptr, st)
-              : fft_dispatch<float, float, FFT_SITE>(blk, blk, L, n_slots, n_rows, 2, false, nullptr, st);
+// x and y fused (one HBM round trip) up to L = 32
+int fft_site_passes(int L) { return L <= 32 ? 2 : 3; }
+
+template <typename R>
+static cudaError_t fft_forward_site(void* blk, int L, int n_slots, int n_rows, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  const bool fused = L <= 32;
+  if (fused) e = fft_xy_site<R, R, false>(blk, L, n_slots, n_rows, st);
+  for (int axis = fused ? 2 : 0; axis < 3 && e == cudaSuccess; axis++)
+    e = fft_dispatch<R, R, FFT_SITE>(blk, blk, L, n_slots, n_rows, axis, false, nullptr, st);
+  return e;
+}
+
+cudaError_t launch_fft_forward_site(void* blk, int L, int n_slots, int n_rows, int kind, cudaStream_t st) {
+  return kind == RK_F64  ? fft_forward_site<double>(blk, L, n_slots, n_rows, st)
+         : kind == RK_DF ? fft_forward_site<dfr>(blk, L, n_slots, n_rows, st)
+                         : fft_forward_site<float>(blk, L, n_slots, n_rows, st);
+}
+
+cudaError_t launch_fft_inverse_site_df(void* ct, void* out, int L, int n_ch, const double* scale, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  if (L <= 32) e = fft_xy_site<dfr, dfr, true>(ct, L, 1, n_ch * 16, st);
+  else
+    for (int axis = 0; axis < 2 && e == cudaSuccess; axis++)
+      e = fft_dispatch<dfr, dfr, FFT_SITE>(ct, ct, L, 1, n_ch * 16, axis, true, nullptr, st);
+  if (e != cudaSuccess) return e;
+  return fft_dispatch<dfr, dfr, FFT_SITE2OUT, double>(ct, out, L, 1, n_ch * 16, 2, true, scale, st);
 }
 
 cudaError_t launch_fft_inverse_site(void* ct, void* out, int L, int n_ch, const double* scale, bool fp64_compute,
@@ -812,7 +964,7 @@ cudaError_t launch_fft_inverse_site(void* ct, void* out, int L, int n_ch, const 
   cudaError_t e;
   if (ct_f32) {  // complex64 q-space correlators, FP32 transform, complex128 output
     if (L <= 32) {
-      e = fft_xy_site<float, float>(ct, L, 1, n_ch * 16, true, st);
+      e = fft_xy_site<float, float, true>(ct, L, 1, n_ch * 16, st);
     } else {
       e = cudaSuccess;
       for (int axis = 0; axis < 2 && e == cudaSuccess; axis++)
@@ -822,8 +974,8 @@ cudaError_t launch_fft_inverse_site(void* ct, void* out, int L, int n_ch, const 
     return fft_dispatch<float, float, FFT_SITE2OUT, double>(ct, out, L, 1, n_ch * 16, 2, true, scale, st);
   }
   if (L <= 32) {
-    e = fp64_compute ? fft_xy_site<double, double>(ct, L, 1, n_ch * 16, true, st)
-                     : fft_xy_site<double, float>(ct, L, 1, n_ch * 16, true, st);
+    e = fp64_compute ? fft_xy_site<double, double, true>(ct, L, 1, n_ch * 16, st)
+                     : fft_xy_site<double, float, true>(ct, L, 1, n_ch * 16, st);
     if (e != cudaSuccess) return e;
   } else {
     for (int axis = 0; axis < 2; axis++) {

@@ -102,7 +102,10 @@ cudaError_t launch_fft_forward_df(const void* blk_site, void* blk_field, int L, 
                                   cudaStream_t st);
 // Forward 3-D FFT in place on site-major blocks blk[slots][V][n_rows] (lanes
 // over the contiguous row index); output is q-major.
-cudaError_t launch_fft_forward_site(void* blk, int L, int n_slots, int n_rows, bool fp64, cudaStream_t st);
+// kind: RK_F32, RK_F64 or RK_DF (storage and arithmetic).
+cudaError_t launch_fft_forward_site(void* blk, int L, int n_slots, int n_rows, int kind, cudaStream_t st);
+// Passes of one such transform, and of launch_fft_inverse_site.
+int fft_site_passes(int L);
 // The forward FP32 transform of launch_fft_forward_site (L <= 32) as one
 // persistent launch over a device work queue (fft.cu): words = [ticket
 // counter, done[tiles]] (fft_queue_ints(L, n_slots, n_rows) ints, zeroed by the
@@ -123,6 +126,8 @@ cudaError_t launch_fft_forward_queue(void* blk, int L, int n_slots, int n_rows, 
 // ct_f32: ct holds complex64 values (then the transform computes in FP32).
 cudaError_t launch_fft_inverse_site(void* ct, void* out, int L, int n_ch, const double* scale, bool fp64_compute,
                                     cudaStream_t st, bool ct_f32 = false);
+// The same from double-float values ct in double-float arithmetic.
+cudaError_t launch_fft_inverse_site_df(void* ct, void* out, int L, int n_ch, const double* scale, cudaStream_t st);
 // Fused FP32 contraction of one slice from q-major blocks blk[V][n_out]: one
 // CTA per pair {q, -q} (qlist[n_q]), block row i staged at shared-memory slot
 // row_slot[i] < n_slots (task offsets are slots), warp units wunits {batch,
@@ -202,6 +207,38 @@ cudaError_t launch_pair_products_df(const void* blk_field, int L, const DevTask*
 cudaError_t launch_wick_sums_df(const void* P, int L, const int* cptr, const int* citem, const float2* ccoef_df,
                                 int n_ch, void* ct, cudaStream_t st);
 cudaError_t launch_fft_inverse_df(void* ct, void* out, int L, int n_ch, const double* scale, cudaStream_t st);
+// Digit-sliced tensor-core contraction (tc_exact.cu) of the FP64 (df = false)
+// and double-float paths, on q-major blocks blk[V][n_out] with products P[V][n_items]:
+// the operands' exponents E[n_q][n_jobs] (one per operand row and q), the
+// products (small tasks one per thread, then the trace set per pair {q, -q} of
+// qlist[n_pairs] and the slice set per q) and the signed sums over Wick diagrams
+// into ct[V][n_outputs].  The mbarrier waits give up after spin_limit polls and
+// set bit 1 of *err.
+constexpr int kExactMaxBlocks = 48;   // blocks of the trace set (its sums and three stages fill shared memory)
+constexpr int kExactMaxSliceA = 128;  // rows of one instruction
+constexpr int kExactMaxSliceB = 32;
+constexpr int kExactSmallSteps = 16;  // open indices of a small task
+struct ExactDev {  // device view of an ExactSet
+  int nA, nB, nAp, nBp, K;
+  const int *rowA, *rowB, *expA, *expB;
+  int n_ent;
+  const int2* entries;  // needed entries: row | column << 16, P item at q | item at -q << 16 (-1: none)
+};
+struct ExactArgs {
+  ExactDev trace, slice;
+  int n_jobs, n_small, n_items;
+  const int *jobs, *small;  // (first row, rows) per exponent job; task ids
+  const DevTask* tasks;
+};
+cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const int* jobs, int n_jobs,
+                                   int* E, cudaStream_t st);
+cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, const ExactArgs& a, const int* E,
+                                  const int* qlist, int n_pairs, void* P, int* err, long long spin_limit,
+                                  cudaStream_t st);
+size_t exact_wick_smem(int n_items);
+cudaError_t launch_exact_wick(const void* P, int V, int n_items, const int* cptr, const int* citem,
+                              const double* ccoef, const float2* ccoef_df, int n_outputs, void* ct, bool df,
+                              cudaStream_t st);
 // ... then the signed FP64 sums over Wick diagrams into ct[n_ch*16][V] (complex128).
 cudaError_t launch_wick_sums(const void* P, int L, const int* cptr, const int* citem, const double* ccoef, int n_ch,
                              void* ct, bool fp64, cudaStream_t st);

@@ -199,6 +199,26 @@ void tc_units(const TcSplit& split, int tiles, std::vector<int>* units);
 // then every task is in rest.  Returns false only on an internal inconsistency.
 bool split_tensor_tasks(const Plan& plan, TcSplit* out, std::string* err);
 
+// Digit-sliced tensor-core products of the FP64-accurate paths (exact_split.cpp).
+// One set is a matrix product per q (or pair {q, -q}): operand row i of A is
+// the field rows rowA[i] .. (its open indices) at q, row j of B at -q; the
+// product (i, j) goes to P item itemQ[i * nBp + j] at q and to itemNQ[...] at -q
+// (-1: not needed).
+struct ExactSet {
+  int nAp = 0, nBp = 0;                // operand rows, padded to 16 (0: the set is empty)
+  std::vector<int> rowA, rowB;         // first field row of each operand row
+  std::vector<int> expA, expB;         // exponent job of each operand row
+  std::vector<short> itemQ, itemNQ;    // [nAp][nBp]
+};
+struct ExactSplit {
+  ExactSet trace, slice;
+  std::vector<int> jobs;               // (first field row, rows) per exponent job
+  std::vector<int> small;              // tasks with few open indices, one product per thread
+  std::vector<char> done;              // per task: its products come from the sets
+  bool all = false;                    // the sets and `small` make every product of the plan
+};
+void make_exact_split(const Plan& plan, ExactSplit* out);
+
 // Partition of the tasks into `groups` lists of near-equal cost (longest task
 // first to the cheapest list); each list is run by one warp for 32 q at a time.
 // by_shape: lists hold tasks of one shape (nA) only and come shape by shape,
