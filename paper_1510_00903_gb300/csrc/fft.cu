@@ -653,11 +653,18 @@ __device__ __forceinline__ void line_fft_cg(const cpx<float>* p, long long step,
   }
 }
 
-// Row-tile width of the queue-driven transform: two plane buffers of
-// N * N * QT complex64 values fit three CTAs per SM.
+// Row-tile width of the queue-driven transform and its plane buffers of
+// N * N * QT complex64 values per CTA: two (the next plane is copied while this
+// one is transformed) where three such CTAs fit an SM with tiles of 64-byte runs
+// or more; at N = 32 one buffer of 8 columns, the other CTAs of the SM covering
+// the copies (32^3, 7368 rows: two buffers of 4 columns took 2.38 ms).
 template <int N>
 __host__ __device__ constexpr int queue_tile() {
-  return N <= 16 ? 16 : (N == 24 ? 8 : 4);
+  return N <= 16 ? 16 : 8;
+}
+template <int N>
+__host__ __device__ constexpr int queue_buffers() {
+  return N <= 24 ? 2 : 1;
 }
 template <int N>
 __host__ __device__ constexpr int queue_line_units() {
@@ -673,7 +680,8 @@ k_fft_site_queue(cpx<float>* __restrict__ data, int n_inner, int tiles_per_outer
   constexpr int U = N + ZU;
   constexpr int PLANE = N * N * TI;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<float>* bufs = reinterpret_cast<cpx<float>*>(smem_raw);  // [2][N * N][TI]
+  constexpr int NBUF = queue_buffers<N>();
+  cpx<float>* bufs = reinterpret_cast<cpx<float>*>(smem_raw);  // [NBUF][N * N][TI]
   __shared__ int s_next, s_ok;
   const long long V = (long long)N * N * N;
   const long long total = (long long)(n_tiles + lag) * U;
@@ -706,14 +714,15 @@ k_fft_site_queue(cpx<float>* __restrict__ data, int n_inner, int tiles_per_outer
   __syncthreads();
   long long cur = s_next;
   int b = 0;
-  fetch_plane(cur, bufs);
+  if (NBUF == 2) fetch_plane(cur, bufs);
   cp_async_commit();
   __syncthreads();
   while (cur >= 0 && cur < total) {
     if (tid == 0) s_next = (*(volatile int*)q.err & 1) ? -1 : atomicAdd(q.words, 1);
     __syncthreads();
     const long long nxt = s_next;
-    fetch_plane(nxt, bufs + (b ^ 1) * PLANE);
+    if (NBUF == 2) fetch_plane(nxt, bufs + (b ^ 1) * PLANE);
+    else fetch_plane(cur, bufs);  // the one buffer: this unit's plane
     cp_async_commit();
     const int st = (int)(cur / U), j = (int)(cur % U);
     if (j < N) {  // plane unit: x and y lines of z plane j of tile st
@@ -723,7 +732,7 @@ k_fft_site_queue(cpx<float>* __restrict__ data, int n_inner, int tiles_per_outer
         const int i0 = (g % tiles_per_outer) * TI, z = j;
         cpx<float>* tile = bufs + b * PLANE;
         cpx<float>* plane = data + (o * V + (long long)z * N * N) * n_inner + i0;
-        cp_async_wait_group<1>();  // this unit's plane has landed (the next one may still fly)
+        cp_async_wait_group<NBUF - 1>();  // this unit's plane has landed (the next one may still fly)
         __syncthreads();
         for (int li = tid; li < N * TI; li += 256) {  // x lines: (y, i)
           const int y = li / TI, i = li - y * TI;
@@ -781,7 +790,7 @@ k_fft_site_queue(cpx<float>* __restrict__ data, int n_inner, int tiles_per_outer
     }
     __syncthreads();  // s_next and the current buffer are reused
     cur = nxt;
-    b ^= 1;
+    b ^= NBUF - 1;
   }
   cp_async_wait_all();  // no copy outlives the CTA
 }
@@ -791,7 +800,7 @@ static cudaError_t fft_site_queue_n(void* data, int n_outer, int n_inner, const 
                                     long long spin_limit, cudaStream_t st) {
   constexpr int TI = queue_tile<N>();
   constexpr int U = N + queue_line_units<N>();
-  const size_t sm = 2 * sizeof(cpx<float>) * N * N * TI;
+  const size_t sm = queue_buffers<N>() * sizeof(cpx<float>) * N * N * TI;
   static int granted[64] = {0};
   static int resident[64] = {0};
   int dev = 0;
@@ -822,7 +831,7 @@ static cudaError_t fft_site_queue_n(void* data, int n_outer, int n_inner, const 
 }
 
 int fft_queue_ints(int L, int n_outer, int n_inner) {
-  const int ti = L <= 16 ? 16 : (L == 24 ? 8 : 4);  // queue_tile
+  const int ti = L <= 16 ? 16 : 8;  // queue_tile
   return 1 + n_outer * ((n_inner + ti - 1) / ti);
 }
 
