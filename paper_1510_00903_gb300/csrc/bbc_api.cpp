@@ -53,8 +53,8 @@ Layout layout(const bbc_ctx* c, int slots) {
   const bbc::Plan& p = c->plan;
   Layout L{};
   size_t o = 0;
-  L.ell_chunk = o; o = align256(o + sizeof(int2) * p.ell_chunk.size());
-  L.ell = o; o = align256(o + sizeof(uint32_t) * p.ell.size());
+  L.ell_chunk = o; o = align256(o + sizeof(int2) * c->ell_chunk.size());
+  L.ell = o; o = align256(o + sizeof(uint32_t) * c->ell.size());
   L.zneed = o; o = align256(o + sizeof(uint32_t) * p.zneed.size());
   L.tasks = o; o = align256(o + sizeof(bbc::DevTask) * p.tasks.size());
   L.group_ptr = o; o = align256(o + sizeof(int) * (kMaxPairGroups + 1));
@@ -438,6 +438,12 @@ bbc_status bbc_create_components(bbc_ctx** ctx, const bbc_lattice* lat, bbc_prec
     delete c;
     return fail(nullptr, BBC_EINVAL, "planner failed");
   }
+  try {
+    bbc::row_terms(c->plan, prec == BBC_FP64, prec == BBC_DF64, &c->ell_chunk, &c->ell);
+  } catch (const std::bad_alloc&) {
+    delete c;
+    return fail(nullptr, BBC_ENOMEM, "host allocation failed while planning");
+  }
   // FP32 blocks from dense entry tuples when the tables and shared memory allow
   if (real_kind(prec) == bbc::RK_F32 && c->plan.groups.size() <= (size_t)bbc::kMaxBuildGroups) {
     std::string derr;
@@ -702,8 +708,8 @@ bbc_status bbc_set_workspace(bbc_ctx* c, void* dev_ptr, size_t bytes, int slices
     c->ex_args.n_items = 16 * (int)p.tasks.size();
   }
   struct Up { void* dst; const void* src; size_t n; } ups[] = {
-      {c->d_ell_chunk, p.ell_chunk.data(), sizeof(int2) * p.ell_chunk.size()},
-      {c->d_ell, p.ell.data(), sizeof(uint32_t) * p.ell.size()},
+      {c->d_ell_chunk, c->ell_chunk.data(), sizeof(int2) * c->ell_chunk.size()},
+      {c->d_ell, c->ell.data(), sizeof(uint32_t) * c->ell.size()},
       {c->d_zneed, p.zneed.data(), sizeof(uint32_t) * p.zneed.size()},
       {c->d_tasks, tasks.data(), sizeof(bbc::DevTask) * tasks.size()},
       {c->d_group_ptr, c->group_ptr.data(), sizeof(int) * c->group_ptr.size()},

@@ -1,6 +1,7 @@
 // ctx_internal.hpp -- definition of the opaque bbc_ctx (internal to libbbc).
 #pragma once
 
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <utility>
@@ -23,6 +24,8 @@ struct bbc_ctx {
   char* ws = nullptr;
   size_t ws_bytes = 0;
   int slots = 0;
+  std::vector<int2> ell_chunk;           // the block rows' terms in device format (row_terms)
+  std::vector<uint32_t> ell;
   int2* d_ell_chunk = nullptr;           // (offset, length) of each 32-row chunk of block rows
   uint32_t* d_ell = nullptr;             // lane-interleaved row entries
   uint32_t* d_zneed = nullptr;
@@ -144,6 +147,46 @@ inline void to_dev_tasks(const PairTask* src, size_t n, const std::vector<int>* 
     d.n2 = t.n2;
     d.sA = t.sA1 | (t.sA2 << 16);
     d.sB = t.sB1 | (t.sB2 << 16);
+  }
+}
+
+// The block-build row terms as the kernels read them: position | weight << 16 with
+// the weight as the top half of an FP32 value (fp64: of an FP64 value).
+// powers: weights that are no power of two become several terms (double-float
+// products are then exact word by word).
+inline void row_terms(const Plan& p, bool fp64, bool powers, std::vector<int2>* chunks, std::vector<uint32_t>* ell) {
+  chunks->clear();
+  ell->clear();
+  auto bits = [&](int w) -> uint32_t {
+    if (fp64) {
+      const double d = w;
+      uint64_t u;
+      std::memcpy(&u, &d, sizeof u);
+      return (uint32_t)(u >> 32) & 0xffff0000u;
+    }
+    const float f = (float)w;
+    uint32_t u;
+    std::memcpy(&u, &f, sizeof u);
+    return u & 0xffff0000u;
+  };
+  for (const auto& c : p.ell_chunk) {
+    std::vector<uint32_t> lane[32];
+    size_t len = 0;
+    for (int l = 0; l < 32; l++) {
+      for (int k = 0; k < c.second; k++) {
+        const uint32_t e = p.ell[c.first + 32 * k + l];
+        const int w = (int)(int16_t)(e >> 16), m = w < 0 ? -w : w;
+        if (w == 0) continue;
+        if (!powers) lane[l].push_back((e & 0xffffu) | bits(w));
+        else
+          for (int b = 0; m >> b; b++)
+            if ((m >> b) & 1) lane[l].push_back((e & 0xffffu) | bits(w < 0 ? -(1 << b) : 1 << b));
+      }
+      len = std::max(len, lane[l].size());
+    }
+    chunks->push_back(make_int2((int)ell->size(), (int)len));
+    for (size_t k = 0; k < len; k++)
+      for (int l = 0; l < 32; l++) ell->push_back(k < lane[l].size() ? lane[l][k] : 0u);  // padding: weight 0 at position 0
   }
 }
 

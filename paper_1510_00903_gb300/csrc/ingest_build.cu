@@ -120,6 +120,91 @@ __constant__ int c_gam[4][4][3] = {{{0, 1, 1}, {1, 0, -1}, {2, 3, 1}, {3, 2, -1}
                                    {{0, 0, 1}, {1, 1, 1}, {2, 2, -1}, {3, 3, -1}},
                                    {{0, 1, 1}, {1, 0, 1}, {2, 3, -1}, {3, 2, -1}}};
 
+// D_{f0 f1}[e0][e1][c2] = sum eps(c0,c1,c2) Gamma1(a0,a1) S_f0[(a0,c0),e0] S_f1[(a1,c1),e1]
+// of `sites` sites: a thread forms the three colours c2 of one (diquark, e0, e1)
+// from the same 24 propagator values (one colour per thread read 48 for the
+// three and spent more on indices than on arithmetic).
+template <typename R, int THREADS>
+__device__ __forceinline__ void diquarks(const cpx<R>* sS, cpx<R>* sD, const DevGroups& g, int sites) {
+  const int per = g.n_dq * 144;
+  for (int ii = threadIdx.x; ii < sites * per; ii += THREADS) {
+    const int s = ii / per, i = ii - s * per, dq = i / 144, e01 = i % 144, e0 = e01 / 12, e1 = e01 % 12;
+    const cpx<R>* S0 = sS + s * 288 + 144 * g.dq_f0[dq] + e0;
+    const cpx<R>* S1 = sS + s * 288 + 144 * g.dq_f1[dq] + e1;
+    const int gam = g.dq_gam[dq];
+    cpx<R> acc[3];
+#pragma unroll
+    for (int gi = 0; gi < 4; gi++) {
+      const bool neg = c_gam[gam][gi][2] < 0;
+      const cpx<R>* p0 = S0 + 36 * c_gam[gam][gi][0];
+      const cpx<R>* p1 = S1 + 36 * c_gam[gam][gi][1];
+      cpx<R> x[3], y[3];
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        x[c] = p0[12 * c];
+        y[c] = p1[12 * c];
+      }
+#pragma unroll
+      for (int c2 = 0; c2 < 3; c2++) {
+        const int ca = (c2 + 1) % 3, cb = (c2 + 2) % 3;  // eps(ca,cb,c2) = +1, eps(cb,ca,c2) = -1
+        if constexpr (std::is_same<R, float>::value) {
+          // the two products rounded before they meet (FP32 results are sensitive to the order)
+          const float sg = neg ? -1.f : 1.f;
+          cpx<R> t(0.f, 0.f), u(0.f, 0.f);
+          if (gi == 0) acc[c2] = cpx<R>(0.f, 0.f);
+          cmac(t, x[ca], y[cb]);
+          cmac(u, x[cb], y[ca]);
+          acc[c2].re += sg * (t.re - u.re);
+          acc[c2].im += sg * (t.im - u.im);
+        } else {
+          const cpx<R> a = neg ? cpx<R>(-x[ca].re, -x[ca].im) : x[ca], b = neg ? x[cb] : cpx<R>(-x[cb].re, -x[cb].im);
+          if (gi == 0) acc[c2] = a * y[cb];
+          else cmac(acc[c2], a, y[cb]);
+          cmac(acc[c2], b, y[ca]);
+        }
+      }
+    }
+#pragma unroll
+    for (int c2 = 0; c2 < 3; c2++) sD[s * 3 * per + 3 * i + c2] = acc[c2];
+  }
+}
+
+// A row term is position | weight << 16, the weight as the top half of an FP32
+// value (FP64: of an FP64 value): one AND gives it, no table.  acc += w z;
+// double-float weights are powers of two (the host splits others), so w z is
+// exact word by word and needs no product error.
+__device__ __forceinline__ float row_add(uint32_t e, float z, float acc) {
+  return fmaf(__uint_as_float(e & 0xffff0000u), z, acc);
+}
+__device__ __forceinline__ dfr row_add(uint32_t e, dfr z, dfr acc) {
+  const float w = __uint_as_float(e & 0xffff0000u);
+  float s, t;
+  two_sum(acc.hi, __fmul_rn(w, z.hi), s, t);
+  return dfr(s, __fadd_rn(t, __fmaf_rn(w, z.lo, acc.lo)));
+}
+__device__ __forceinline__ double row_add(uint32_t e, double z, double acc) {
+  return ::fma(__hiloint2double((int)(e & 0xffff0000u), 0), z, acc);
+}
+// the row of this lane in a chunk (lane-interleaved terms ep[32 k], k < len), for
+// SITES sites `zs` positions apart
+template <typename R, int SITES>
+__device__ __forceinline__ void row_sum(const cpx<R>* sZ, int zs, const uint32_t* ep, int len, cpx<R> (&acc)[SITES]) {
+#pragma unroll
+  for (int s = 0; s < SITES; s++) acc[s] = cpx<R>(0, 0);
+  for (int k = 0; k < len; k++) {
+    const uint32_t e = __ldg(ep + 32 * k);  // padding: weight 0 at position 0
+    // FP64 is bound by its narrow pipe: skip the padding's multiply-adds
+    // there; the other types run them (no divergent branch)
+    if (std::is_same<R, double>::value && (e >> 16) == 0) continue;
+#pragma unroll
+    for (int s = 0; s < SITES; s++) {
+      const cpx<R> z = sZ[s * zs + (e & 0xffffu)];
+      acc[s].re = row_add(e, z.re, acc[s].re);
+      acc[s].im = row_add(e, z.im, acc[s].im);
+    }
+  }
+}
+
 // One CTA builds the blocks of SITES consecutive sites with THREADS threads:
 // the propagators, diquarks and tensor entries of every site sit in shared
 // memory, and each thread runs one block row for all SITES sites, so every
@@ -134,38 +219,15 @@ k_block_build(const cpx<R>* __restrict__ prop, int V, const int2* __restrict__ e
   cpx<R>* sS = reinterpret_cast<cpx<R>*>(smem_raw);  // [SITES][2][144]  light, strange
   cpx<R>* sD = sS + SITES * 288;                      // [SITES][n_dq][432]  the diquarks the families read
   cpx<R>* sZ = sD + SITES * nd;                       // [SITES][g.z_slots] the tensor entries the rows read
-  R* sW = reinterpret_cast<R*>(sZ + SITES * g.z_slots);  // weights -16..15 (no int->float conversion per term)
   const int site0 = blockIdx.x * SITES, slot = blockIdx.y, tid = threadIdx.x;
   const int zs = g.z_slots;
-  if (tid < 32) sW[tid] = (R)(tid - 16);
   const cpx<R>* P = prop + (size_t)slot * 2 * V * 144;
   for (int i = tid; i < SITES * 288; i += THREADS) {
     const int s = i / 288, j = i - s * 288;
     sS[i] = P[(size_t)(j / 144) * V * 144 + (size_t)(site0 + s) * 144 + j % 144];
   }
   __syncthreads();
-  // D_{f0 f1}[e0][e1][c2] = sum eps(c0,c1,c2) Gamma1(a0,a1) S_f0[(a0,c0),e0] S_f1[(a1,c1),e1]
-  for (int ii = tid; ii < SITES * nd; ii += THREADS) {
-    const int s = ii / nd, i = ii - s * nd;
-    const int dq = i / 432, r = i % 432, e0 = r / 36, e1 = (r / 3) % 12, c2 = r % 3;
-    const int ca = (c2 + 1) % 3, cb = (c2 + 2) % 3;  // eps(ca,cb,c2) = +1, eps(cb,ca,c2) = -1
-    const cpx<R>* S0 = sS + s * 288 + 144 * g.dq_f0[dq];
-    const cpx<R>* S1 = sS + s * 288 + 144 * g.dq_f1[dq];
-    const int gam = g.dq_gam[dq];
-    cpx<R> acc(0, 0);
-#pragma unroll
-    for (int gi = 0; gi < 4; gi++) {
-      const int a0 = c_gam[gam][gi][0], a1 = c_gam[gam][gi][1];
-      const R sg = (R)c_gam[gam][gi][2];
-      cpx<R> t(0, 0);
-      cmac(t, S0[(3 * a0 + ca) * 12 + e0], S1[(3 * a1 + cb) * 12 + e1]);
-      cpx<R> u(0, 0);
-      cmac(u, S0[(3 * a0 + cb) * 12 + e0], S1[(3 * a1 + ca) * 12 + e1]);
-      acc.re += sg * (t.re - u.re);
-      acc.im += sg * (t.im - u.im);
-    }
-    sD[ii] = acc;
-  }
+  diquarks<R, THREADS>(sS, sD, g, SITES);
   __syncthreads();
   for (int gi = 0; gi < g.n; gi++) {
     // the tensor entries this group reads (and the previous group did not leave)
@@ -180,8 +242,10 @@ k_block_build(const cpx<R>* __restrict__ prop, int V, const int2* __restrict__ e
       const cpx<R>* S2 = sS + s * 288 + 144 * g.fam_f2[fam];
       const int a = i / 1728 + g.spin0, r = i % 1728, e01 = r / 12, e2 = r % 12;
       cpx<R> acc(0, 0);
-#pragma unroll
-      for (int c2 = 0; c2 < 3; c2++) cmac(acc, D[e01 * 3 + c2], S2[(3 * a + c2) * 12 + e2]);
+      if constexpr (std::is_same<R, dfr>::value) acc = D[e01 * 3] * S2[36 * a + e2];  // no sums with zero
+      else cmac(acc, D[e01 * 3], S2[36 * a + e2]);
+      cmac(acc, D[e01 * 3 + 1], S2[36 * a + 12 + e2]);
+      cmac(acc, D[e01 * 3 + 2], S2[36 * a + 24 + e2]);
       sZ[s * zs + pos] = acc;
     }
     __syncthreads();
@@ -190,25 +254,8 @@ k_block_build(const cpx<R>* __restrict__ prop, int V, const int2* __restrict__ e
     for (int r = r0 + tid; r < r1; r += THREADS) {
       // the warp's 32 rows are one chunk: entry k of all of them is 128 contiguous bytes
       const int2 ch = __ldg(ell_chunk + g.chunk_first[gi] + ((r - r0) >> 5));
-      const uint32_t* ep = ell + ch.x + ((r - r0) & 31);
       cpx<R> acc[SITES];
-#pragma unroll
-      for (int s = 0; s < SITES; s++) acc[s] = cpx<R>(0, 0);
-      for (int k = 0; k < ch.y; k++) {
-        const uint32_t e = __ldg(ep + 32 * k);  // padding: weight 0 at position 0
-        // FP64 is bound by its narrow pipe: skip the padding's multiply-adds
-        // there; the other types run them (no divergent branch)
-        if constexpr (sizeof(R) == 8 && std::is_floating_point<R>::value)
-          if ((e >> 16) == 0) continue;
-        const R w = sW[((int)(int16_t)(e >> 16)) + 16];
-        const int pos = e & 0xffffu;
-#pragma unroll
-        for (int s = 0; s < SITES; s++) {
-          const cpx<R> z = sZ[s * zs + pos];
-          acc[s].re = fma(w, z.re, acc[s].re);
-          acc[s].im = fma(w, z.im, acc[s].im);
-        }
-      }
+      row_sum<R, SITES>(sZ, zs, ell + ch.x + ((r - r0) & 31), ch.y, acc);
 #pragma unroll
       for (int s = 0; s < SITES; s++) out[(size_t)s * n_out + r] = acc[s];
     }
@@ -244,27 +291,7 @@ k_block_build_dense(const cpx<float>* __restrict__ prop, int V, const int2* __re
     }
   }
   __syncthreads();
-  for (int ii = tid; ii < SITES * nd; ii += kThreads) {
-    const int s = ii / nd, i = ii - s * nd;
-    const int dq = i / 432, r = i % 432, e0 = r / 36, e1 = (r / 3) % 12, c2 = r % 3;
-    const int ca = (c2 + 1) % 3, cb = (c2 + 2) % 3;  // eps(ca,cb,c2) = +1, eps(cb,ca,c2) = -1
-    const cpx<float>* S0 = sS + s * 288 + 144 * g.dq_f0[dq];
-    const cpx<float>* S1 = sS + s * 288 + 144 * g.dq_f1[dq];
-    const int gam = g.dq_gam[dq];
-    cpx<float> acc(0.f, 0.f);
-#pragma unroll
-    for (int gi = 0; gi < 4; gi++) {
-      const int a0 = c_gam[gam][gi][0], a1 = c_gam[gam][gi][1];
-      const float sg = (float)c_gam[gam][gi][2];
-      cpx<float> t(0.f, 0.f);
-      cmac(t, S0[(3 * a0 + ca) * 12 + e0], S1[(3 * a1 + cb) * 12 + e1]);
-      cpx<float> u(0.f, 0.f);
-      cmac(u, S0[(3 * a0 + cb) * 12 + e0], S1[(3 * a1 + ca) * 12 + e1]);
-      acc.re += sg * (t.re - u.re);
-      acc.im += sg * (t.im - u.im);
-    }
-    sD[ii] = acc;
-  }
+  diquarks<float, THREADS>(sS, sD, g, SITES);
   __syncthreads();
   for (int gi = 0; gi < g.n; gi++) {
     const int t0 = g.tuple_first[gi], nt = g.tuple_first[gi + 1] - t0, str = g.stride[gi];
@@ -276,36 +303,29 @@ k_block_build_dense(const cpx<float>* __restrict__ prop, int V, const int2* __re
       const cpx<float>* D = sD + s * nd + 432 * g.fam_dq[fam] + 3 * e01;
       const cpx<float>* S2 = sS + s * 288 + 144 * g.fam_f2[fam] + 36 * (a + g.spin0);
       const cpx<float> d0 = D[0], d1 = D[1], d2 = D[2];
+      const float4* S4 = reinterpret_cast<const float4*>(S2);  // two columns per load
       cpx<float>* z = sZ + s * zs + j;
 #pragma unroll
-      for (int e2 = 0; e2 < 12; e2++) {
-        cpx<float> acc(0.f, 0.f);
-        cmac(acc, d0, S2[e2]);
-        cmac(acc, d1, S2[12 + e2]);
-        cmac(acc, d2, S2[24 + e2]);
-        z[e2 * str] = acc;
+      for (int e2 = 0; e2 < 12; e2 += 2) {
+        const float4 x0 = S4[e2 / 2], x1 = S4[6 + e2 / 2], x2 = S4[12 + e2 / 2];
+        cpx<float> a0(0.f, 0.f), a1(0.f, 0.f);
+        cmac(a0, d0, cpx<float>(x0.x, x0.y));
+        cmac(a1, d0, cpx<float>(x0.z, x0.w));
+        cmac(a0, d1, cpx<float>(x1.x, x1.y));
+        cmac(a1, d1, cpx<float>(x1.z, x1.w));
+        cmac(a0, d2, cpx<float>(x2.x, x2.y));
+        cmac(a1, d2, cpx<float>(x2.z, x2.w));
+        z[e2 * str] = a0;
+        z[(e2 + 1) * str] = a1;
       }
     }
     __syncthreads();
     const int r0 = g.first[gi], r1 = r0 + g.rows[gi];
     cpx<float>* out = blk + ((size_t)slot * V + site0) * n_out;
     for (int r = r0 + tid; r < r1; r += kThreads) {
-      cpx<float> acc[SITES];
-#pragma unroll
-      for (int s = 0; s < SITES; s++) acc[s] = cpx<float>(0.f, 0.f);
       const int2 ch = __ldg(ell_chunk + g.dchunk_first[gi] + ((r - r0) >> 5));
-      const uint32_t* ep = ell + ch.x + ((r - r0) & 31);
-      for (int k = 0; k < ch.y; k++) {
-        const uint32_t e = __ldg(ep + 32 * k);  // padding: weight 0 at position 0
-        const float w = __uint_as_float(e & 0xffff0000u);
-        const int pos = e & 0xffffu;
-#pragma unroll
-        for (int s = 0; s < SITES; s++) {
-          const cpx<float> zv = sZ[s * zs + pos];
-          acc[s].re = fmaf(w, zv.re, acc[s].re);
-          acc[s].im = fmaf(w, zv.im, acc[s].im);
-        }
-      }
+      cpx<float> acc[SITES];
+      row_sum<float, SITES>(sZ, zs, ell + ch.x + ((r - r0) & 31), ch.y, acc);
 #pragma unroll
       for (int s = 0; s < SITES; s++) out[(size_t)s * n_out + r] = acc[s];
     }
@@ -350,7 +370,7 @@ cudaError_t launch_block_build_dense(const void* prop, int V, int n_slots, const
 
 size_t block_build_smem(int z_slots, int sites, bool fp64, int n_dq) {  // fp64: 8-byte reals (FP64 or double-float)
   const size_t cb = fp64 ? sizeof(cpx<double>) : sizeof(cpx<float>);
-  return (size_t)sites * (288 + 432 * (size_t)n_dq + z_slots) * cb + 32 * (fp64 ? sizeof(double) : sizeof(float));
+  return (size_t)sites * (288 + 432 * (size_t)n_dq + z_slots) * cb;
 }
 
 bool build_variant_supported(int sites, int threads) {

@@ -42,8 +42,8 @@ StaticLayout static_layout(const bbc_ctx* c) {
   const size_t cb = c->prec == BBC_FP64 ? 16 : 8, V = (size_t)c->V;
   StaticLayout L{};
   size_t o = 0;
-  L.ell_chunk = o; o = a256(o + sizeof(int2) * p.ell_chunk.size());
-  L.ell = o; o = a256(o + sizeof(uint32_t) * p.ell.size());
+  L.ell_chunk = o; o = a256(o + sizeof(int2) * c->ell_chunk.size());
+  L.ell = o; o = a256(o + sizeof(uint32_t) * c->ell.size());
   L.zneed = o; o = a256(o + sizeof(uint32_t) * p.zneed.size());
   L.tasks = o; o = a256(o + sizeof(bbc::DevTask) * p.tasks.size());
   L.group_ptr = o; o = a256(o + sizeof(int) * c->group_ptr.size());
@@ -117,8 +117,8 @@ extern "C" bbc_status bbc_run_slice_static(bbc_ctx* c, int t, const void* S_ligh
   cudaStream_t st = c->stream;
   // plan tables (copies from pageable host memory return once the data is staged)
   struct Up { size_t off; const void* src; size_t n; } ups[] = {
-      {L.ell_chunk, p.ell_chunk.data(), sizeof(int2) * p.ell_chunk.size()},
-      {L.ell, p.ell.data(), sizeof(uint32_t) * p.ell.size()},
+      {L.ell_chunk, c->ell_chunk.data(), sizeof(int2) * c->ell_chunk.size()},
+      {L.ell, c->ell.data(), sizeof(uint32_t) * c->ell.size()},
       {L.zneed, p.zneed.data(), sizeof(uint32_t) * p.zneed.size()},
       {L.group_ptr, c->group_ptr.data(), sizeof(int) * c->group_ptr.size()},
       {L.group_task, c->group_task.data(), sizeof(int) * c->group_task.size()},
