@@ -462,7 +462,7 @@ bbc_status bbc_create_components(bbc_ctx** ctx, const bbc_lattice* lat, bbc_prec
       delete c;
       return fail(nullptr, BBC_ENOMEM, "host allocation failed while scheduling");
     }
-    c->exact = c->ex.all && bbc::exact_wick_smem(16 * (int)c->plan.tasks.size()) <= bbc::kMaxSmemPerBlock;
+    c->exact = c->ex.all && bbc::exact_wick_fits(16 * (int)c->plan.tasks.size(), (int)c->ex.wick_coefs.size());
   }
   // warp task groups of the pair products: enough warps per 32 q to fill the
   // GPU several times over at L = 16 (V/32 q tiles x groups warps); the
@@ -877,8 +877,7 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
     }
     {
       StageScope scope(c, BBC_STAGE_WICK);
-      e = c->exact ? bbc::launch_exact_wick(c->d_P, c->V, c->ex_args.n_items, c->d_cptr, c->d_citem, c->d_ccoef,
-                                            c->d_ccoef_df, n_ch * 16, c->d_ct, c->prec == BBC_DF64, c->stream)
+      e = c->exact ? bbc::launch_exact_wick(c->d_P, c->V, c->ex_args, c->prec == BBC_DF64, n_ch * 16, c->d_ct, c->stream)
           : c->prec == BBC_DF64
               ? bbc::launch_wick_sums_df(c->d_P, c->lat.L, c->d_cptr, c->d_citem, c->d_ccoef_df, n_ch, c->d_ct,
                                          c->stream)

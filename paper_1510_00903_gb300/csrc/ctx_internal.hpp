@@ -190,8 +190,8 @@ inline void row_terms(const Plan& p, bool fp64, bool powers, std::vector<int2>* 
   }
 }
 
-// Device tables of the digit-sliced sets, packed into one array of ints: jobs
-// and small tasks, then per set rowA, rowB, expA, expB and the needed entries (padded to 16
+// Device tables of the digit-sliced contraction, packed into one array of ints:
+// jobs and small tasks, the Wick sums, then per set rowA, rowB, expA, expB and the needed entries (padded to 16
 // bytes); *a points into it at `base`.
 inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, ExactArgs* a) {
   std::vector<int> t;
@@ -205,15 +205,27 @@ inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, Exact
   a->n_small = (int)s.small.size();
   a->jobs = put(s.jobs.data(), sizeof(int) * s.jobs.size());
   a->small = put(s.small.data(), sizeof(int) * s.small.size());
-  const ExactSet* sets[2] = {&s.trace, &s.slice};
-  for (int i = 0; i < 2; i++) {
-    const ExactSet& x = *sets[i];
-    ExactDev& d = i == 0 ? a->trace : a->slice;
+  WickDev& w = a->wick;
+  w.n_chunks = (int)s.wick_chunks.size();
+  w.n_coefs = (int)s.wick_coefs.size();
+  w.chunks = (const int2*)put(s.wick_chunks.data(), sizeof(int2) * s.wick_chunks.size());
+  w.outputs = (const int2*)put(s.wick_outputs.data(), sizeof(int2) * s.wick_outputs.size());
+  w.ell = (const uint32_t*)put(s.wick_ell.data(), sizeof(uint32_t) * s.wick_ell.size());
+  w.coefs = (const double*)put(s.wick_coefs.data(), sizeof(double) * s.wick_coefs.size());
+  std::vector<float> split;
+  for (double x : s.wick_coefs) {
+    split.push_back((float)x);
+    split.push_back((float)(x - (double)(float)x));
+  }
+  w.coefs_df = (const float2*)put(split.data(), sizeof(float) * split.size());
+  for (int i = 0; i < kExactSets; i++) {
+    const ExactSet& x = s.set[i];
+    ExactDev& d = a->set[i];
     d.nA = (int)x.rowA.size();
     d.nB = (int)x.rowB.size();
     d.nAp = x.nAp;
     d.nBp = x.nBp;
-    d.K = i == 0 ? 144 : 36;
+    d.K = i < kExactSlice ? 144 : 36;
     d.rowA = put(x.rowA.data(), sizeof(int) * x.rowA.size());
     d.rowB = put(x.rowB.data(), sizeof(int) * x.rowB.size());
     d.expA = put(x.expA.data(), sizeof(int) * x.expA.size());
@@ -232,6 +244,7 @@ inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, Exact
   return t;
 }
 
+static_assert(sizeof(std::pair<int, int>) == sizeof(int2), "pairs are uploaded as int2");
 static_assert(N_DIQUARK == kMaxDiquarks && N_FAMILY == kMaxFamilies && kMaxGroups == kMaxBuildGroups,
               "diquark, family and group tables");
 

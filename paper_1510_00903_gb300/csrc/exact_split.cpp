@@ -1,18 +1,21 @@
-// exact_split.cpp -- which block-pair products of the FP64-accurate paths run
-// as digit-sliced tensor-core products (tc_exact.cu).
+// exact_split.cpp -- which block-pair products run as digit-sliced tensor-core
+// products (tc_exact.cu).
 //
-// Two task forms of the planner (Sec. 3 Eq. LN.pLLp.FFT) are matrix products
-// whose operands are shared by many tasks:
-//   trace form (4 x 4 spins, 12 x 12 open indices): tr(M_A(q) M_B(-q)) of whole
-//     12 x 12 blocks, over all such blocks one nb x nb product of 144 terms;
-//     G(-q) = G(q)^T, so one product serves a pair {q, -q};
-//   slice form (8 x 2 or 2 x 8 spins, 12 x 3 open indices): 36 consecutive rows
-//     of one block against 36 of another, one nA x nB product per q.
+// Most tasks of the planner (Sec. 3 Eq. LN.pLLp.FFT) have forms that are matrix
+// products whose operands are shared by many tasks:
+//   trace forms (4 x 4 spins, 12 x 12 open indices): sums over whole 12 x 12
+//     blocks, tr(M_A(q) M_B(-q)) or the same without the transpose, over all such
+//     blocks one nb x nb product of 144 terms; G(-q) = G(q)^T, so one product
+//     serves a pair {q, -q};
+//   slice forms (8 x 2 or 2 x 8 spins, 12 x 3 open indices): 36 consecutive rows
+//     of one block (or three columns of it) against 36 consecutive rows of
+//     another, one nA x nB product per q.
 // Every product the tasks need gets its place in the product buffer P through
 // the item tables; tasks with few open indices are made one product per thread.
 // A plan with any other task (or more operands than the kernel holds) keeps the
-// CUDA-core products of field-major blocks.
+// CUDA-core products.
 #include <algorithm>
+#include <iterator>
 #include <map>
 #include <set>
 
@@ -23,98 +26,107 @@ namespace bbc {
 
 namespace {
 
-constexpr int kTraceForm[6] = {12, 12, 12, 1, 1, 12};  // n1, n2, sA1, sA2, sB1, sB2
-constexpr int kSliceForm[6] = {12, 3, 1, 12, 1, 12};
+// n1, n2, sA1, sA2, sB1, sB2
+constexpr int kTraceForms[2][6] = {{12, 12, 12, 1, 1, 12}, {12, 12, 12, 1, 12, 1}};
+// slices, seen from the 8-spin side: both of consecutive rows, or the 8-side of columns
+constexpr int kSliceForms[2][6] = {{12, 3, 1, 12, 1, 12}, {12, 3, 12, 1, 1, 12}};
 
-bool has_form(const PairTask& t, const int (&f)[6]) {
-  return t.n1 == f[0] && t.n2 == f[1] && t.sA1 == f[2] && t.sA2 == f[3] && t.sB1 == f[4] && t.sB2 == f[5];
+bool has_form(const PairTask& t, const int (&f)[6], bool swapped) {
+  return t.n1 == f[0] && t.n2 == f[1] && (swapped ? t.sB1 : t.sA1) == f[2] && (swapped ? t.sB2 : t.sA2) == f[3] &&
+         (swapped ? t.sA1 : t.sB1) == f[4] && (swapped ? t.sA2 : t.sB2) == f[5];
 }
 
 int index_of(const std::vector<int>& v, int x) { return (int)(std::lower_bound(v.begin(), v.end(), x) - v.begin()); }
 
-}  // namespace
-
-void make_exact_split(const Plan& plan, ExactSplit* out) {
-  ExactSplit S;
+// trace form f: operands, item tables, done tasks
+void trace_set(const Plan& plan, int f, ExactSet* T, std::vector<char>* done) {
   const int n = (int)plan.tasks.size();
-  S.done.assign(n, 0);
-  *out = ExactSplit();
-  if (n * 16 > 32767) return;  // the item tables hold 16-bit indices
-  // trace form
+  auto is = [&](const PairTask& t) { return t.nA == 4 && t.nB == 4 && has_form(t, kTraceForms[f], false); };
   std::set<int> blocks;
   for (const PairTask& t : plan.tasks)
-    if (t.nA == 4 && t.nB == 4 && has_form(t, kTraceForm))
+    if (is(t))
       for (int r = 0; r < 4; r++) {
         blocks.insert(t.offA[r]);
         blocks.insert(t.offB[r]);
       }
-  ExactSet& T = S.trace;
-  if (!blocks.empty() && (int)blocks.size() <= kExactMaxBlocks) {
-    T.rowA.assign(blocks.begin(), blocks.end());
-    T.rowB = T.rowA;
-    T.nAp = T.nBp = ((int)blocks.size() + 15) / 16 * 16;
-    T.itemQ.assign((size_t)T.nAp * T.nBp, -1);
-    for (int ti = 0; ti < n; ti++) {
-      const PairTask& t = plan.tasks[ti];
-      if (!(t.nA == 4 && t.nB == 4 && has_form(t, kTraceForm))) continue;
-      std::vector<size_t> at;
-      for (int ra = 0; ra < 4; ra++)
-        for (int rb = 0; rb < 4; rb++) at.push_back((size_t)index_of(T.rowA, t.offA[ra]) * T.nBp + index_of(T.rowB, t.offB[rb]));
-      bool free_all = std::set<size_t>(at.begin(), at.end()).size() == 16;
-      for (size_t a : at) free_all &= T.itemQ[a] < 0;
-      if (!free_all) continue;  // a second task on the same products stays on the CUDA cores
-      for (int i = 0; i < 16; i++) T.itemQ[at[i]] = (short)(16 * ti + i);
-      S.done[ti] = 1;
-    }
-    T.itemNQ.assign(T.itemQ.size(), -1);
-    for (int i = 0; i < T.nAp; i++)
-      for (int j = 0; j < T.nBp; j++) T.itemNQ[(size_t)i * T.nBp + j] = T.itemQ[(size_t)j * T.nBp + i];
+  if (blocks.empty() || (int)blocks.size() > kExactMaxBlocks) return;
+  T->rowA.assign(blocks.begin(), blocks.end());
+  T->rowB = T->rowA;
+  T->nAp = T->nBp = ((int)blocks.size() + 15) / 16 * 16;
+  T->itemQ.assign((size_t)T->nAp * T->nBp, -1);
+  for (int ti = 0; ti < n; ti++) {
+    const PairTask& t = plan.tasks[ti];
+    if (!is(t)) continue;
+    std::set<size_t> seen;
+    std::vector<size_t> at;
+    bool free_all = true;
+    for (int ra = 0; ra < 4; ra++)
+      for (int rb = 0; rb < 4; rb++) {
+        at.push_back((size_t)index_of(T->rowA, t.offA[ra]) * T->nBp + index_of(T->rowB, t.offB[rb]));
+        free_all &= T->itemQ[at.back()] < 0 && seen.insert(at.back()).second;
+      }
+    if (!free_all) continue;  // a second task on the same products: not for this kernel
+    for (int i = 0; i < 16; i++) T->itemQ[at[i]] = (short)(16 * ti + i);
+    (*done)[ti] = 1;
   }
-  // slice form: the 8-side's rows are A, the 2-side's B; a 2 x 8 task reads B at
-  // q and A at -q, so its product belongs to the place of -q
-  auto slice = [&](const PairTask& t, const int** a8, const int** b2, bool* swapped) {
-    if (!has_form(t, kSliceForm) || !((t.nA == 8 && t.nB == 2) || (t.nA == 2 && t.nB == 8))) return false;
-    *swapped = t.nA == 2;
+  T->itemNQ.assign(T->itemQ.size(), -1);
+  for (int i = 0; i < T->nAp; i++)
+    for (int j = 0; j < T->nBp; j++) T->itemNQ[(size_t)i * T->nBp + j] = T->itemQ[(size_t)j * T->nBp + i];
+}
+
+// slice form f: the 8-side's rows are A, the 2-side's B; a 2 x 8 task reads B at
+// q and A at -q, so its product belongs to the place of -q
+void slice_set(const Plan& plan, int f, ExactSet* C, std::vector<char>* done) {
+  const int n = (int)plan.tasks.size();
+  auto is = [&](const PairTask& t, const int** a8, const int** b2, bool* swapped) {
+    *swapped = t.nA == 2 && t.nB == 8;
+    if (!(*swapped || (t.nA == 8 && t.nB == 2)) || !has_form(t, kSliceForms[f], *swapped)) return false;
     *a8 = *swapped ? t.offB : t.offA;
     *b2 = *swapped ? t.offA : t.offB;
     return true;
   };
   std::set<int> rowsA, rowsB;
-  for (const PairTask& t : plan.tasks) {
-    const int *a8, *b2;
-    bool sw;
-    if (!slice(t, &a8, &b2, &sw)) continue;
-    rowsA.insert(a8, a8 + 8);
-    rowsB.insert(b2, b2 + 2);
-  }
-  ExactSet& C = S.slice;
-  if (!rowsA.empty() && (int)rowsA.size() <= kExactMaxSliceA && (int)rowsB.size() <= kExactMaxSliceB) {
-    C.rowA.assign(rowsA.begin(), rowsA.end());
-    C.rowB.assign(rowsB.begin(), rowsB.end());
-    C.nAp = ((int)rowsA.size() + 15) / 16 * 16;
-    C.nBp = ((int)rowsB.size() + 15) / 16 * 16;
-    C.itemQ.assign((size_t)C.nAp * C.nBp, -1);
-    C.itemNQ.assign((size_t)C.nAp * C.nBp, -1);
-    for (int ti = 0; ti < n; ti++) {
-      const PairTask& t = plan.tasks[ti];
-      const int *a8, *b2;
-      bool sw;
-      if (!slice(t, &a8, &b2, &sw)) continue;
-      std::vector<short>& items = sw ? C.itemNQ : C.itemQ;
-      bool free_all = true;
-      std::set<size_t> seen;
-      for (int a = 0; a < 8; a++)
-        for (int b = 0; b < 2; b++) {
-          const size_t at = (size_t)index_of(C.rowA, a8[a]) * C.nBp + index_of(C.rowB, b2[b]);
-          free_all &= items[at] < 0 && seen.insert(at).second;
-        }
-      if (!free_all) continue;
-      for (int a = 0; a < 8; a++)
-        for (int b = 0; b < 2; b++)
-          items[(size_t)index_of(C.rowA, a8[a]) * C.nBp + index_of(C.rowB, b2[b])] =
-              (short)(16 * ti + (sw ? b * 8 + a : a * 2 + b));
-      S.done[ti] = 1;
+  const int *a8, *b2;
+  bool sw;
+  for (const PairTask& t : plan.tasks)
+    if (is(t, &a8, &b2, &sw)) {
+      rowsA.insert(a8, a8 + 8);
+      rowsB.insert(b2, b2 + 2);
     }
+  if (rowsA.empty() || (int)rowsA.size() > kExactMaxSliceA || (int)rowsB.size() > kExactMaxSliceB) return;
+  C->rowA.assign(rowsA.begin(), rowsA.end());
+  C->rowB.assign(rowsB.begin(), rowsB.end());
+  C->nAp = ((int)rowsA.size() + 15) / 16 * 16;
+  C->nBp = ((int)rowsB.size() + 15) / 16 * 16;
+  C->itemQ.assign((size_t)C->nAp * C->nBp, -1);
+  C->itemNQ.assign((size_t)C->nAp * C->nBp, -1);
+  for (int ti = 0; ti < n; ti++) {
+    if (!is(plan.tasks[ti], &a8, &b2, &sw)) continue;
+    std::vector<short>& items = sw ? C->itemNQ : C->itemQ;
+    std::set<size_t> seen;
+    bool free_all = true;
+    auto at = [&](int a, int b) { return (size_t)index_of(C->rowA, a8[a]) * C->nBp + index_of(C->rowB, b2[b]); };
+    for (int a = 0; a < 8; a++)
+      for (int b = 0; b < 2; b++) free_all &= items[at(a, b)] < 0 && seen.insert(at(a, b)).second;
+    if (!free_all) continue;
+    for (int a = 0; a < 8; a++)
+      for (int b = 0; b < 2; b++) items[at(a, b)] = (short)(16 * ti + (sw ? b * 8 + a : a * 2 + b));
+    (*done)[ti] = 1;
+  }
+}
+
+}  // namespace
+
+void make_exact_split(const Plan& plan, ExactSplit* out) {
+  constexpr int align = 2;  // field rows per 32 bytes: operands are read in such pieces
+  ExactSplit S;
+  const int n = (int)plan.tasks.size();
+  std::vector<char> done(n, 0);
+  *out = ExactSplit();
+  if (n * 16 > 32767) return;  // the item tables hold 16-bit indices
+  for (int f = 0; f < 2; f++) {
+    trace_set(plan, f, &S.set[kExactTrace + f], &done);
+    slice_set(plan, f, &S.set[kExactSlice + f], &done);
   }
   // exponent jobs (first row, rows): one per trace block, and one per slice that
   // lies in no trace block (a slice inside one shares its exponent)
@@ -128,30 +140,68 @@ void make_exact_split(const Plan& plan, ExactSplit* out) {
     job_of[{first, rows}] = id;
     return id;
   };
-  for (int r : T.rowA) T.expA.push_back(job(r, 144));
-  T.expB = T.expA;
-  auto slice_job = [&](int r) {
-    auto it = std::upper_bound(T.rowA.begin(), T.rowA.end(), r);
-    if (it != T.rowA.begin() && r + 36 <= *(it - 1) + 144) return job(*(it - 1), 144);
-    return job(r, 36);
+  std::set<int> blocks;
+  bool ok = plan.n_out % align == 0;
+  for (int f = 0; f < 2; f++) {
+    ExactSet& T = S.set[f];
+    for (int r : T.rowA) {
+      blocks.insert(r);
+      T.expA.push_back(job(r, 144));
+      ok &= r % align == 0;
+    }
+    T.expB = T.expA;
+  }
+  auto slice_job = [&](int r, int len) {
+    auto it = blocks.upper_bound(r);
+    if (it != blocks.begin() && r + len <= *std::prev(it) + 144) return job(*std::prev(it), 144);
+    return job(r, len);
   };
-  for (int r : C.rowA) C.expA.push_back(slice_job(r));
-  for (int r : C.rowB) C.expB.push_back(slice_job(r));
+  for (int f = 0; f < 2; f++) {
+    ExactSet& C = S.set[kExactSlice + f];
+    // rows an operand spans: 36, or 11 x 12 + 3 for three columns of a block
+    const int lenA = f == 0 ? 36 : 135;
+    for (int r : C.rowA) {
+      C.expA.push_back(slice_job(r, lenA));
+      ok &= f == 1 || r % align == 0;
+    }
+    for (int r : C.rowB) {
+      C.expB.push_back(slice_job(r, 36));
+      ok &= r % align == 0;
+    }
+  }
   if (S.jobs.empty()) return;
-  // every operand row lies inside the block rows, at an even row (32-byte loads)
-  bool ok = plan.n_out % 2 == 0;
-  auto inside = [&](const std::vector<int>& rows, int len) {
-    for (int r : rows) ok &= r >= 0 && r % 2 == 0 && r + len <= plan.n_out;
-  };
-  inside(T.rowA, 144);
-  inside(C.rowA, 36);
-  inside(C.rowB, 36);
+  // every operand row lies inside the block rows
+  for (size_t j = 0; j < S.jobs.size(); j += 2) ok &= S.jobs[j] >= 0 && S.jobs[j] + S.jobs[j + 1] <= plan.n_out;
   for (int ti = 0; ti < n; ti++) {
     const PairTask& t = plan.tasks[ti];
-    if (S.done[ti]) continue;
+    if (done[ti]) continue;
     if (t.n1 * t.n2 > kExactSmallSteps) return;
     S.small.push_back(ti);
   }
+  // signed sums
+  const int n_o = (int)plan.tcontrib_ptr.size() - 1;
+  std::vector<int> order(n_o);
+  for (int o = 0; o < n_o; o++) order[o] = o;
+  auto terms = [&](int o) { return plan.tcontrib_ptr[o + 1] - plan.tcontrib_ptr[o]; };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return terms(a) > terms(b); });
+  std::map<double, int> coef_of;
+  for (int c0 = 0; c0 < n_o; c0 += 32) {
+    const int len = terms(order[c0]), base = (int)S.wick_ell.size();
+    S.wick_chunks.push_back({base, len});
+    S.wick_ell.resize(base + 32 * (size_t)len, 0u);
+    for (int l = 0; l < 32; l++) {
+      const int o = c0 + l < n_o ? order[c0 + l] : -1, nt = o < 0 ? 0 : terms(o);
+      S.wick_outputs.push_back({o, nt});
+      for (int k = 0; k < nt; k++) {
+        const double x = plan.tcontrib_coef[plan.tcontrib_ptr[o] + k];
+        auto it = coef_of.emplace(x, (int)S.wick_coefs.size());
+        if (it.second) S.wick_coefs.push_back(x);
+        S.wick_ell[base + 32 * (size_t)k + l] =
+            (uint32_t)plan.tcontrib_item[plan.tcontrib_ptr[o] + k] | ((uint32_t)it.first->second << 16);
+      }
+    }
+  }
+  ok &= S.wick_coefs.size() <= 65536;
   S.all = ok;
   *out = std::move(S);
 }

@@ -210,22 +210,35 @@ cudaError_t launch_fft_inverse_df(void* ct, void* out, int L, int n_ch, const do
 // Digit-sliced tensor-core contraction (tc_exact.cu) of the FP64 (df = false)
 // and double-float paths, on q-major blocks blk[V][n_out] with products P[V][n_items]:
 // the operands' exponents E[n_q][n_jobs] (one per operand row and q), the
-// products (small tasks one per thread, then the trace set per pair {q, -q} of
-// qlist[n_pairs] and the slice set per q) and the signed sums over Wick diagrams
-// into ct[V][n_outputs].  The mbarrier waits give up after spin_limit polls and
-// set bit 1 of *err.
-constexpr int kExactMaxBlocks = 48;   // blocks of the trace set (its sums and three stages fill shared memory)
+// products (small tasks one product per thread, then the trace sets per pair
+// {q, -q} of qlist[n_pairs] and the slice sets per q) and the signed sums over
+// Wick diagrams into ct[V][n_outputs].  The mbarrier waits give up after
+// spin_limit polls and set bit 1 of *err.
+constexpr int kExactMaxBlocks = 48;   // blocks of a trace set (its sums and three stages fill shared memory)
 constexpr int kExactMaxSliceA = 128;  // rows of one instruction
 constexpr int kExactMaxSliceB = 32;
 constexpr int kExactSmallSteps = 16;  // open indices of a small task
+constexpr int kExactSets = 4;
+// forms of a set: trace tr(M_A M_B), the same without the transpose, slices of
+// 36 consecutive rows, slices whose A side is three columns of a block
+enum { kExactTrace = 0, kExactSame = 1, kExactSlice = 2, kExactSliceT = 3 };
 struct ExactDev {  // device view of an ExactSet
   int nA, nB, nAp, nBp, K;
   const int *rowA, *rowB, *expA, *expB;
   int n_ent;
   const int2* entries;  // needed entries: row | column << 16, P item at q | item at -q << 16 (-1: none)
 };
+struct WickDev {  // signed sums: outputs sorted by length, 32 per chunk, lane-interleaved terms
+  int n_chunks, n_coefs;
+  const int2* chunks;       // offset into ell, terms of the longest output
+  const int2* outputs;      // [32 n_chunks] output (-1: none), its terms
+  const uint32_t* ell;      // P item | coefficient index << 16
+  const double* coefs;      // the distinct coefficients, and split into two FP32 words
+  const float2* coefs_df;
+};
 struct ExactArgs {
-  ExactDev trace, slice;
+  ExactDev set[kExactSets];  // by form
+  WickDev wick;
   int n_jobs, n_small, n_items;
   const int *jobs, *small;  // (first row, rows) per exponent job; task ids
   const DevTask* tasks;
@@ -235,9 +248,8 @@ cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int 
 cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, const ExactArgs& a, const int* E,
                                   const int* qlist, int n_pairs, void* P, int* err, long long spin_limit,
                                   cudaStream_t st);
-size_t exact_wick_smem(int n_items);
-cudaError_t launch_exact_wick(const void* P, int V, int n_items, const int* cptr, const int* citem,
-                              const double* ccoef, const float2* ccoef_df, int n_outputs, void* ct, bool df,
+bool exact_wick_fits(int n_items, int n_coefs);
+cudaError_t launch_exact_wick(const void* P, int V, const ExactArgs& a, bool df, int n_outputs, void* ct,
                               cudaStream_t st);
 // ... then the signed FP64 sums over Wick diagrams into ct[n_ch*16][V] (complex128).
 cudaError_t launch_wick_sums(const void* P, int L, const int* cptr, const int* citem, const double* ccoef, int n_ch,

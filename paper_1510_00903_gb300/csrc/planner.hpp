@@ -199,11 +199,10 @@ void tc_units(const TcSplit& split, int tiles, std::vector<int>* units);
 // then every task is in rest.  Returns false only on an internal inconsistency.
 bool split_tensor_tasks(const Plan& plan, TcSplit* out, std::string* err);
 
-// Digit-sliced tensor-core products of the FP64-accurate paths (exact_split.cpp).
-// One set is a matrix product per q (or pair {q, -q}): operand row i of A is
-// the field rows rowA[i] .. (its open indices) at q, row j of B at -q; the
-// product (i, j) goes to P item itemQ[i * nBp + j] at q and to itemNQ[...] at -q
-// (-1: not needed).
+// Digit-sliced tensor-core products (exact_split.cpp).  One set is a matrix
+// product per q (or pair {q, -q}): operand row i of A is the field rows rowA[i] ..
+// (its open indices) at q, row j of B at -q; the product (i, j) goes to P item
+// itemQ[i * nBp + j] at q and to itemNQ[...] at -q (-1: not needed).
 struct ExactSet {
   int nAp = 0, nBp = 0;                // operand rows, padded to 16 (0: the set is empty)
   std::vector<int> rowA, rowB;         // first field row of each operand row
@@ -211,11 +210,16 @@ struct ExactSet {
   std::vector<short> itemQ, itemNQ;    // [nAp][nBp]
 };
 struct ExactSplit {
-  ExactSet trace, slice;
+  ExactSet set[4];                     // by form: kExactTrace .. kExactSliceT (kernels.cuh)
   std::vector<int> jobs;               // (first field row, rows) per exponent job
   std::vector<int> small;              // tasks with few open indices, one product per thread
-  std::vector<char> done;              // per task: its products come from the sets
   bool all = false;                    // the sets and `small` make every product of the plan
+  // signed sums over Wick diagrams: outputs sorted by length, 32 per chunk, entry k
+  // of the chunk's lane l at ell[chunk.first + 32 k + l] = P item | coefficient << 16
+  std::vector<std::pair<int, int>> wick_chunks;   // offset, terms of the longest output
+  std::vector<std::pair<int, int>> wick_outputs;  // 32 per chunk: output (-1: none), its terms
+  std::vector<uint32_t> wick_ell;
+  std::vector<double> wick_coefs;                 // the distinct coefficients
 };
 void make_exact_split(const Plan& plan, ExactSplit* out);
 

@@ -25,8 +25,8 @@
 // On field-major blocks (16-byte loads 64 KB and more apart) the same kernel was
 // TLB bound at 0.98 and 45 ms: the blocks are q-major for it.
 //
-// Two operand sets (exact_split.cpp):
-//   trace form, one product per pair {q, -q}: STACK = 2.  Two digit slices of
+// Operand sets (exact_split.cpp):
+//   trace forms, one product per pair {q, -q}: STACK = 2.  Two digit slices of
 //     A (nbp <= 64 rows each) fill one M = 128 instruction, so a window that
 //     starts at slice i gives level i + j in its first nbp rows of D and
 //     i + j + 1 in the next nbp: four column blocks hold the eight levels.
@@ -35,7 +35,7 @@
 //     Windows at even i take the even digits, at odd i (from -1, a slice of
 //     zeros in front) the odd ones, so every digit pair up to level 7 is met
 //     once.
-//   slice form, one product per q: STACK = 1.  The window is one slice (up to
+//   slice forms, one product per q: STACK = 1.  The window is one slice (up to
 //     128 rows), all eight levels are column blocks of nB columns, and digit i
 //     of A meets digits 0 .. 7 - i of B in one instruction.
 // Re = Re Re - Im Im uses the instruction's negated A.
@@ -63,7 +63,7 @@ constexpr int kXDigits = 8;
 constexpr int kXWarps = 20;
 constexpr int kXEpi = 8;                       // epilogue warps (tensor-memory lanes 32 (w mod 4) .., column chunks w / 4)
 constexpr int kXProd = kXWarps - kXEpi - 1;    // producer warps, after the MMA warp
-constexpr int kXMaxStages = 8;
+constexpr int kXMaxStages = 6;
 constexpr int kXCols = 512;                    // all of tensor memory: one CTA per SM
 constexpr int kXFixed = 2048;                  // static shared memory (at most)
 constexpr int kXBad = 0x7fffffff;              // exponent of a row with a NaN or infinite value
@@ -182,8 +182,8 @@ __device__ __forceinline__ unsigned long long x_fix(dfr x, int e) {
   const float y = __fmaf_rn(x.lo, __fmul_rn(s, p17), r1);
   const float t2 = __fadd_rn(y, M), r2 = __fsub_rn(y, __fsub_rn(t2, M));
   const float t3 = __fmaf_rn(r2, p17, M);
-  constexpr long long Mb = 0x4B400000;
-  constexpr unsigned long long off = kXBias - (unsigned long long)(((Mb << 17) + 2 * Mb) * 131072 + Mb);
+  constexpr unsigned long long Mb = 0x4B400000;
+  constexpr unsigned long long off = kXBias - (((Mb << 17) + 2 * Mb) * 131072 + Mb);
   const unsigned long long hi =
       (unsigned long long)__float_as_uint(t0) * 131072u + (unsigned long long)__float_as_uint(t1) + __float_as_uint(t2);
   // (the mask: a row with infinities has any digits)
@@ -290,10 +290,36 @@ __device__ __forceinline__ long long x_mad(unsigned a, unsigned b, long long c) 
   return d;
 }
 __device__ __forceinline__ long long x_int(uint32_t x) { return (long long)__float2int_rn(__uint_as_float(x) * 1048576.f); }
-// weights 2^42, 2^28, 2^14, 1 (shift 0: the even levels) or 2^35, 2^21, 2^7, 2^-7 (the odd ones)
-__device__ __forceinline__ long long x_sum4(long long n0, long long n1, long long n2, long long n3, bool even) {
-  const long long e = (n0 << 28) + (n1 << 14) + n2;
-  return even ? (e << 14) + n3 : (e << 7) + (n3 >> 7);
+// Sum over the levels of column j, weights 2^(42 - 7 s) (the last one, 2^-7, cut).
+// STACK 2: a[c] is level 2 c (even) or 2 c + 1; STACK 1: level c.
+__device__ __forceinline__ long long x_levels(const uint32_t (&a)[4][4], int j, bool even, uint32_t& wide) {
+  constexpr long long off = kXMagic * ((1ll << 28) + (1ll << 14) + 1);
+  const unsigned n0 = x_bits(a[0][j], wide), n1 = x_bits(a[1][j], wide), n2 = x_bits(a[2][j], wide);
+  const int n3 = (int)(x_bits(a[3][j], wide) - (unsigned)kXMagic);
+  const long long v = x_mad(n0, 1u << 28, x_mad(n1, 1u << 14, n2)) - off;
+  return (v << (even ? 14 : 7)) + (n3 >> (even ? 0 : 7));
+}
+__device__ __forceinline__ long long x_levels(const uint32_t (&a)[8][4], int j, bool, uint32_t& wide) {
+  constexpr long long off = kXMagic * ((1ll << 28) + (1ll << 14) + 1);
+  const unsigned n0 = x_bits(a[0][j], wide), n1 = x_bits(a[1][j], wide), n2 = x_bits(a[2][j], wide);
+  const unsigned n3 = x_bits(a[3][j], wide), n4 = x_bits(a[4][j], wide), n5 = x_bits(a[5][j], wide);
+  const int n6 = (int)(x_bits(a[6][j], wide) - (unsigned)kXMagic);
+  const int n7 = (int)(x_bits(a[7][j], wide) - (unsigned)kXMagic);
+  const long long ev = x_mad(n0, 1u << 28, x_mad(n2, 1u << 14, n4)) - off;
+  const long long od = x_mad(n1, 1u << 28, x_mad(n3, 1u << 14, n5)) - off;
+  return (ev << 14) + n6 + (od << 7) + (n7 >> 7);
+}
+// the same for sums beyond 2^22
+template <int NC>
+__device__ __forceinline__ long long x_levels_wide(const uint32_t (&a)[NC][4], int j, bool even) {
+  long long v = 0;
+#pragma unroll
+  for (int c = 0; c < NC; c++) {
+    const int s = NC == 4 ? 2 * c + (even ? 0 : 1) : c, sh = 42 - 7 * s;
+    const long long n = x_int(a[c][j]);
+    v += sh >= 0 ? n << (sh & 63) : n >> (-sh & 63);
+  }
+  return v;
 }
 
 // two neighbouring complex values with one 32-byte load (32-byte aligned)
@@ -306,8 +332,9 @@ __device__ __forceinline__ void x_load2(const float4* p, double2& a, double2& b)
   asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a.x), "=d"(a.y), "=d"(b.x), "=d"(b.y) : "l"(p));
 }
 
+// Per block type: a loaded complex value and its parts.
 template <typename T>
-struct XRaw;  // a loaded complex value: re, im
+struct XRaw;
 template <>
 struct XRaw<double> {
   using load = double2;
@@ -320,6 +347,17 @@ struct XRaw<dfr> {
   static __device__ __forceinline__ dfr re(const float4& v) { return dfr(v.x, v.y); }
   static __device__ __forceinline__ dfr im(const float4& v) { return dfr(v.z, v.w); }
 };
+// values j .. j + 3 from four neighbouring elements
+template <typename Ld>
+__device__ __forceinline__ void x_run4(const Ld* p, Ld (&v)[8], int j) {
+  x_load2(reinterpret_cast<const float4*>(p), v[j], v[j + 1]);
+  x_load2(reinterpret_cast<const float4*>(p + 2), v[j + 2], v[j + 3]);
+}
+// values j and j + 4 from two neighbouring elements
+template <typename Ld>
+__device__ __forceinline__ void x_pair(const Ld* p, Ld (&v)[8], int j) {
+  x_load2(reinterpret_cast<const float4*>(p), v[j], v[j + 4]);
+}
 
 struct XShape {  // shared-memory layout of one launch
   int slA, slB, partA, stage, n_stages, off_b, sums, bytes;  // sums: the epilogue's 64-bit sums, after the stages
@@ -343,26 +381,27 @@ __host__ __device__ inline XShape x_shape(int stack, int nAp, int nBp) {
 // Exponents of one q per CTA: E[q][job] with max |component| over the job's
 // rows below 0.985 2^E (kXBad: a NaN or infinite value among them); a warp per
 // job, one pass over the operand rows: HBM bound.
+__device__ __forceinline__ int x_mag(const double2& v) {  // the exponent-carrying words
+  return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+}
+__device__ __forceinline__ int x_mag(const float4& v) {  // both words of a double-float count
+  return max(__float_as_int(fabsf(v.x) + fabsf(v.y)) & 0x7fffffff, __float_as_int(fabsf(v.z) + fabsf(v.w)) & 0x7fffffff);
+}
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_exact_exponents(const float4* __restrict__ F, int n_out, const int* __restrict__ jobs, int n_jobs,
+k_exact_exponents(const void* __restrict__ blk, int n_out, const int* __restrict__ jobs, int n_jobs,
                   int* __restrict__ E) {
+  using Ld = typename XRaw<T>::load;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float4* row = F + (size_t)blockIdx.x * n_out;
+  const Ld* row = reinterpret_cast<const Ld*>(blk) + (size_t)blockIdx.x * n_out;
   for (int job = warp; job < n_jobs; job += 8) {
     const int first = __ldg(jobs + 2 * job), rows = __ldg(jobs + 2 * job + 1);
     int m = 0;
 #pragma unroll 5
-    for (int r = lane; r < rows; r += 32) {
-      const float4 v = __ldg(row + first + r);
-      // the exponent-carrying words of re and im; double-float: both words count
-      const float x = std::is_same<T, double>::value ? v.y : fabsf(v.x) + fabsf(v.y);
-      const float y = std::is_same<T, double>::value ? v.w : fabsf(v.z) + fabsf(v.w);
-      m = max(m, max(__float_as_int(x) & 0x7fffffff, __float_as_int(y) & 0x7fffffff));
-    }
+    for (int r = lane; r < rows; r += 32) m = max(m, x_mag(__ldg(row + first + r)));
     m = __reduce_max_sync(0xffffffffu, m);
     // 2^-5 of headroom in the significand: the largest magnitude has to fit
-    // eight digits whose range is [-64, 63]; a row of zeros or subnormals counts as zero
+    // digits whose range is [-64, 63]; a row of zeros or subnormals counts as zero
     int e;
     if (std::is_same<T, double>::value) e = m >= 0x7ff00000 ? kXBad : m < 0x100000 ? 0 : ((m + 0x8000) >> 20) - 1022;
     else e = m >= 0x7f800000 ? kXBad : max(((m + 0x40000) >> 23) - 126, -72);
@@ -370,140 +409,154 @@ k_exact_exponents(const float4* __restrict__ F, int n_out, const int* __restrict
   }
 }
 
+// Product i of a task with few open indices, from the rows of q and -q.
+__device__ __forceinline__ double2 x_small(const double2* a, const double2* c, int n1, int n2, int sA1, int sA2, int sB1,
+                                           int sB2) {
+  cpx<double> acc(0, 0);
+  for (int i1 = 0; i1 < n1; i1++)
+    for (int i2 = 0; i2 < n2; i2++) {
+      const double2 x = __ldg(a + i1 * sA1 + i2 * sA2), y = __ldg(c + i1 * sB1 + i2 * sB2);
+      cmac(acc, cpx<double>(x.x, x.y), cpx<double>(y.x, y.y));
+    }
+  return make_double2(acc.re, acc.im);
+}
+__device__ __forceinline__ float4 x_small(const float4* a, const float4* c, int n1, int n2, int sA1, int sA2, int sB1,
+                                          int sB2) {
+  df64acc re{0.f, 0.f}, im{0.f, 0.f};
+  for (int i1 = 0; i1 < n1; i1++)
+    for (int i2 = 0; i2 < n2; i2++) {
+      const float4 x = __ldg(a + i1 * sA1 + i2 * sA2), y = __ldg(c + i1 * sB1 + i2 * sB2);
+      df_mac(re, x.x, x.y, y.x, y.y);
+      df_mac(re, -x.z, -x.w, y.z, y.w);
+      df_mac(im, x.x, x.y, y.z, y.w);
+      df_mac(im, x.z, x.w, y.x, y.y);
+    }
+  df_renorm(re);
+  df_renorm(im);
+  return make_float4(re.s, re.e, im.s, im.e);
+}
+template <typename Ld>
+__device__ __forceinline__ Ld x_small_item(const Ld* F, int q, int nq, int n_out, const DevTask& t, int i) {
+  const int nB = t.nAnB >> 8;
+  return x_small(F + (size_t)q * n_out + t.offA[i / nB], F + (size_t)nq * n_out + t.offB[i % nB], t.n1, t.n2,
+                 t.sA & 0xffff, t.sA >> 16, t.sB & 0xffff, t.sB >> 16);
+}
+
 // Products of the tasks with few open indices (a few percent of the work): one
 // CTA per q, one product per thread.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_exact_small(const float4* __restrict__ F, int L, int n_out, const DevTask* __restrict__ tasks,
-              const int* __restrict__ small, int n_small, int n_items, float4* __restrict__ P) {
+k_exact_small(const void* __restrict__ blk, int L, int n_out, const DevTask* __restrict__ tasks,
+              const int* __restrict__ small, int n_small, int n_items, void* __restrict__ P) {
+  using Ld = typename XRaw<T>::load;
   const int q = blockIdx.x, nq = x_neg_site(q, L);
   for (int u = threadIdx.x; u < n_small * 16; u += 256) {
     const int ti = __ldg(small + (u >> 4)), i = u & 15;
-    const DevTask& t = tasks[ti];
-    const int nB = t.nAnB >> 8;
-    const float4* a = F + (size_t)q * n_out + t.offA[i / nB];
-    const float4* c = F + (size_t)nq * n_out + t.offB[i % nB];
-    const int sA1 = t.sA & 0xffff, sA2 = t.sA >> 16, sB1 = t.sB & 0xffff, sB2 = t.sB >> 16;
-    float4* out = P + (size_t)q * n_items + ti * 16 + i;
-    if constexpr (std::is_same<T, double>::value) {
-      cpx<double> acc(0, 0);
-      for (int i1 = 0; i1 < t.n1; i1++)
-        for (int i2 = 0; i2 < t.n2; i2++) {
-          const double2 x = __ldg((const double2*)(a + i1 * sA1 + i2 * sA2));
-          const double2 y = __ldg((const double2*)(c + i1 * sB1 + i2 * sB2));
-          cmac(acc, cpx<double>(x.x, x.y), cpx<double>(y.x, y.y));
-        }
-      *(double2*)out = make_double2(acc.re, acc.im);
-    } else {
-      df64acc re{0.f, 0.f}, im{0.f, 0.f};
-      for (int i1 = 0; i1 < t.n1; i1++)
-        for (int i2 = 0; i2 < t.n2; i2++) {
-          const float4 x = __ldg(a + i1 * sA1 + i2 * sA2);
-          const float4 y = __ldg(c + i1 * sB1 + i2 * sB2);
-          df_mac(re, x.x, x.y, y.x, y.y);
-          df_mac(re, -x.z, -x.w, y.z, y.w);
-          df_mac(im, x.x, x.y, y.z, y.w);
-          df_mac(im, x.z, x.w, y.x, y.y);
-        }
-      df_renorm(re);
-      df_renorm(im);
-      *out = make_float4(re.s, re.e, im.s, im.e);
-    }
+    reinterpret_cast<Ld*>(P)[(size_t)q * n_items + ti * 16 + i] =
+        x_small_item(reinterpret_cast<const Ld*>(blk), q, nq, n_out, tasks[ti], i);
   }
 }
 
 // Signed sums over Wick diagrams of q-major products, ct[q][o] = sum_c coef_c
-// P[q][item_c]: one CTA per kWickQ values of q stages their product rows in
-// shared memory, so that every product is read once and the term lists once
-// per kWickQ.  FP64, or double-float with the coefficients split on the host,
-// renormalised every 16 terms.
-constexpr int kWickQ = 2, kWickThreads = 512;
-template <typename T, typename C>
+// P[q][item_c]: one CTA per q stages its product row and the distinct
+// coefficients in shared memory (several CTAs per SM, so that one's copies overlap
+// another's sums).  A warp takes 32 outputs of
+// nearly equal length (host-sorted); their terms are stored lane by lane (item |
+// coefficient index << 16), so a term of 32 outputs is one 128-byte load.  With
+// the outputs' term lists read in place, 7 to 14 cache lines per load, the sums
+// took 93 us (double-float, 16^3, 52 channels).
+// FP64; double-float with the coefficients split on the host, renormalised
+// every 16 terms.
+constexpr int kWickThreads = 256;
+struct WickAcc64 {
+  double x = 0, y = 0;
+  __device__ __forceinline__ void add(double w, double2 v) {
+    x = fma(w, v.x, x);
+    y = fma(w, v.y, y);
+  }
+  __device__ __forceinline__ void renorm() {}
+  __device__ __forceinline__ double2 value() { return make_double2(x, y); }
+};
+struct WickAccDf {
+  df64acc re{0.f, 0.f}, im{0.f, 0.f};
+  __device__ __forceinline__ void add(float2 w, float4 v) {
+    df_mac(re, w.x, w.y, v.x, v.y);
+    df_mac(im, w.x, w.y, v.z, v.w);
+  }
+  __device__ __forceinline__ void renorm() {
+    df_renorm(re);
+    df_renorm(im);
+  }
+  __device__ __forceinline__ float4 value() {
+    renorm();
+    return make_float4(re.s, re.e, im.s, im.e);
+  }
+};
+template <typename T, typename C, typename Acc>
 __global__ void __launch_bounds__(kWickThreads)
-k_exact_wick(const float4* __restrict__ P, int V, int n_items, const int* __restrict__ cptr,
-             const int* __restrict__ citem, const C* __restrict__ ccoef, int n_outputs, float4* __restrict__ ct) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float4* s_p = reinterpret_cast<float4*>(smem);  // [kWickQ][n_items]
-  const int q0 = blockIdx.x * kWickQ, nq = min(kWickQ, V - q0);
-  for (int i = threadIdx.x; i < nq * n_items; i += kWickThreads) cp_async16(s_p + i, P + (size_t)q0 * n_items + i);
-  cp_async_wait_all();
+k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* __restrict__ coefs, int n_outputs,
+             void* __restrict__ ct) {
+  using Ld = typename XRaw<T>::load;
+  extern __shared__ __align__(128) unsigned char smem[];
+  Ld* s_p = reinterpret_cast<Ld*>(smem);                                // [n_items]
+  C* s_c = reinterpret_cast<C*>(smem + (size_t)n_items * sizeof(Ld));  // [n_coefs]
+  const int q = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  {
+    const Ld* src = reinterpret_cast<const Ld*>(P) + (size_t)q * n_items;
+    for (int i = threadIdx.x; i < n_items; i += kWickThreads) cp_async16(s_p + i, src + i);
+    for (int i = threadIdx.x; i < W.n_coefs; i += kWickThreads) s_c[i] = __ldg(coefs + i);
+    cp_async_wait_all();
+  }
   __syncthreads();
-  for (int u = threadIdx.x; u < nq * n_outputs; u += kWickThreads) {
-    const int k = u / n_outputs, o = u - k * n_outputs;
-    const float4* p = s_p + (size_t)k * n_items;
-    const int c0 = __ldg(cptr + o), c1 = __ldg(cptr + o + 1);
-    float4* out = ct + (size_t)(q0 + k) * n_outputs + o;
-    if constexpr (std::is_same<T, double>::value) {
-      double2 s = make_double2(0.0, 0.0);
-      for (int c = c0; c < c1; c += 4) {  // four terms' coefficients and products on their way together
-        C w[4];
-        float4 v[4];
+  for (int c = warp; c < W.n_chunks; c += kWickThreads / 32) {
+    const Ld* p = s_p;
+    const int2 ch = __ldg(W.chunks + c);  // offset, terms of the longest output
+    const int2 out = __ldg(W.outputs + 32 * c + lane);  // output (-1: none), its terms
+    const uint32_t* ep = W.ell + ch.x + lane;
+    Acc acc;
+    for (int j0 = 0; j0 < ch.y; j0 += 4) {  // four terms and their products on their way together
+      uint32_t e[4];
+      Ld v[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-          const int cj = min(c + j, c1 - 1);
-          w[j] = __ldg(ccoef + cj);
-          v[j] = p[__ldg(citem + cj)];
-        }
+      for (int j = 0; j < 4; j++) e[j] = __ldg(ep + 32 * min(j0 + j, ch.y - 1));
 #pragma unroll
-        for (int j = 0; j < 4; j++)
-          if (c + j < c1) {
-            const double2 x = *reinterpret_cast<const double2*>(&v[j]);
-            s.x = fma(w[j], x.x, s.x);
-            s.y = fma(w[j], x.y, s.y);
-          }
-      }
-      *reinterpret_cast<double2*>(out) = s;
-    } else {
-      df64acc re{0.f, 0.f}, im{0.f, 0.f};
-      for (int c = c0; c < c1; c += 4) {
-        C w[4];
-        float4 v[4];
+      for (int j = 0; j < 4; j++) v[j] = p[e[j] & 0xffffu];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-          const int cj = min(c + j, c1 - 1);
-          w[j] = __ldg(ccoef + cj);
-          v[j] = p[__ldg(citem + cj)];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-          if (c + j < c1) {
-            df_mac(re, w[j].x, w[j].y, v[j].x, v[j].y);
-            df_mac(im, w[j].x, w[j].y, v[j].z, v[j].w);
-          }
-        if (((c - c0) & 12) == 12) {  // every 16 terms
-          df_renorm(re);
-          df_renorm(im);
-        }
-      }
-      df_renorm(re);
-      df_renorm(im);
-      *out = make_float4(re.s, re.e, im.s, im.e);
+      for (int j = 0; j < 4; j++)
+        if (j0 + j < out.y) acc.add(s_c[e[j] >> 16], v[j]);
+      if ((j0 & 12) == 12) acc.renorm();  // every 16 terms
     }
+    if (out.x >= 0) reinterpret_cast<Ld*>(ct)[(size_t)q * n_outputs + out.x] = acc.value();
   }
 }
 
 struct XShared {
-  uint64_t bars[2][2 * kXMaxStages + 5];  // one set per operand set
+  uint64_t bars[kExactSets][2 * kXMaxStages + 5];  // one group per operand set
   uint32_t tmem;
   int abort;
-  int ex[2][kExactMaxSliceA], ey[2][kExactMaxBlocks];  // exponents of the product's operand rows, by parity
+  short ex[2][kExactMaxSliceA], ey[2][kExactMaxBlocks];  // exponents of the product's operand rows, by parity
 };
 static_assert(sizeof(XShared) <= kXFixed && kExactMaxBlocks >= kExactMaxSliceB && kExactMaxSliceA >= kExactMaxBlocks,
               "exponents of either set");
 
 // One operand set: the products of qlist[n_q] (nullptr: q = 0 .. n_q - 1).
-template <typename T, int STACK>
-__device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, const float4* __restrict__ F, int L,
+template <typename T, int FORM>
+__device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, const void* __restrict__ blk, int L,
                                           int n_out, const ExactDev& S, const int* __restrict__ E, int n_jobs,
-                                          const int* __restrict__ qlist, int n_q, float4* __restrict__ P,
+                                          const int* __restrict__ qlist, int n_q, void* __restrict__ P,
                                           int n_items, long long spin_limit) {
-  uint64_t* bars = xs.bars[STACK - 1];
+  constexpr int STACK = FORM < kExactSlice ? 2 : 1;
+  using Raw = XRaw<T>;
+  using Ld = typename Raw::load;
+  constexpr int ND = kXDigits;
+  const Ld* F = reinterpret_cast<const Ld*>(blk);
+  uint64_t* bars = xs.bars[FORM];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const XShape sh = x_shape(STACK, S.nAp, S.nBp);
   const int NS = sh.n_stages, NB = S.nBp, nC = (S.K + 15) / 16;
   const int TA = S.nAp / 16, TT = TA + NB / 16;  // warp tasks per stage: 16 rows x 2 k-groups each
   const int n_mine = (n_q - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
-  const int bufW = (STACK == 2 ? 8 : 16) * NB, n_buf = 2 * bufW <= kXCols ? 2 : 1;
+  const int bufW = (STACK == 2 ? ND : 2 * ND) * NB, n_buf = 2 * bufW <= kXCols ? 2 : 1;
   const uint32_t bar_full = x_smem(bars), bar_empty = bar_full + 8 * kXMaxStages;
   const uint32_t bar_acc = bar_empty + 8 * kXMaxStages, bar_free = bar_acc + 16, bar_drain = bar_free + 16;
   if (tid == 0) {
@@ -536,7 +589,6 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
 
   if (warp > kXEpi) {
     // ------------------------------------------------------- producers
-    using Raw = XRaw<T>;
     // Warp tasks in order: product i, chunk c of 16 open indices, then 16 operand
     // rows (A's, then B's) x 2 groups of 8 indices; warp pw takes every kXProd-th.
     struct Cursor {
@@ -566,7 +618,7 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       }
       return true;
     };
-    typename Raw::load v[8];
+    Ld v[8];
     int e = 0;
     auto load = [&](const Cursor& t) {
       const bool sideB = t.w >= TA;
@@ -574,33 +626,37 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       const int q = sideB ? t.nq : t.q;
       e = 0;
 #pragma unroll
-      for (int j = 0; j < 8; j++) v[j] = typename Raw::load();
+      for (int j = 0; j < 8; j++) v[j] = Ld();
       if (row < (sideB ? S.nB : S.nA)) {
-        const float4* p = F + (size_t)q * n_out + __ldg((sideB ? S.rowB : S.rowA) + row);
+        const Ld* p = F + (size_t)q * n_out + __ldg((sideB ? S.rowB : S.rowA) + row);
         e = __ldg(E + (size_t)q * n_jobs + __ldg((sideB ? S.expB : S.expA) + row));
         e = e == kXBad ? 0 : e;  // any digits: the epilogue writes NaN
         if (STACK == 2) {
           // chunk c is the 4 x 4 tile (u, v) = (4 tu .., 4 tv ..) of the open
           // indices, k-group kg its u = 4 tu + 2 kg + (0, 1): values j = 4 du + dv
-          // are element 12 u + v of A's block and element 12 v + u of B's
+          // are element 12 u + v of A's block and of B's, or 12 v + u of B's (transposed)
           const int tu = t.c / 3, tv = t.c - 3 * tu;
-          if (sideB) {
+          if (FORM == kExactTrace && sideB) {
             p += 48 * tv + 4 * tu + 2 * kg;
 #pragma unroll
-            for (int dv = 0; dv < 4; dv++) x_load2(p + 12 * dv, v[dv], v[4 + dv]);
+            for (int dv = 0; dv < 4; dv++) x_pair(p + 12 * dv, v, dv);
           } else {
             p += 48 * tu + 24 * kg + 4 * tv;
-#pragma unroll
-            for (int du = 0; du < 2; du++) {
-              x_load2(p + 12 * du, v[4 * du], v[4 * du + 1]);
-              x_load2(p + 12 * du + 2, v[4 * du + 2], v[4 * du + 3]);
-            }
+            x_run4(p, v, 0);
+            x_run4(p + 12, v, 4);
           }
         } else {
           const int k0 = 16 * t.c + 8 * kg;
+          if (FORM == kExactSliceT && !sideB) {  // k = 12 i2 + i1 is element 12 i1 + i2
 #pragma unroll
-          for (int j = 0; j < 8; j += 2)
-            if (k0 + j < S.K) x_load2(p + k0 + j, v[j], v[j + 1]);  // K is even
+            for (int j = 0; j < 8; j++) {
+              const int k = k0 + j, i2 = k / 12;
+              if (k < S.K) v[j] = __ldg(p + 12 * (k - 12 * i2) + i2);
+            }
+          } else {
+            if (k0 < S.K) x_run4(p + k0, v, 0);  // K is a multiple of 4
+            if (k0 + 4 < S.K) x_run4(p + k0 + 4, v, 4);
+          }
         }
       }
     };
@@ -630,8 +686,8 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       for (int part = 0; part < 2; part++) {
         if (sideB) {
           // STACK 2: even digits, then odd digits
-          x_store_digits(u[part], dst + sh.off_b + part * kXDigits * sh.slB, [&](int d) {
-            return (STACK == 2 ? (d & 1) * (kXDigits / 2) + (d >> 1) : d) * sh.slB;
+          x_store_digits(u[part], dst + sh.off_b + part * ND * sh.slB, [&](int d) {
+            return (STACK == 2 ? (d & 1) * (ND / 2) + (d >> 1) : d) * sh.slB;
           });
         } else {
           x_store_digits(u[part], dst + part * sh.partA + (STACK == 2 ? sh.slA : 0), [&](int d) { return d * sh.slA; });
@@ -646,21 +702,21 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
     // registers; one elected thread issues.  Per window: offsets of its first A
     // and B slice in descriptor units, its first accumulator column, its
     // instructions' descriptors.
-    uint32_t wa[8], wb[8], wn[8];
-    int wc[8];
+    uint32_t wa[ND], wb[ND], wn[ND];
+    int wc[ND];
 #pragma unroll
-    for (int w = 0; w < 8; w++) {
+    for (int w = 0; w < ND; w++) {
       // STACK 2: slices of A count from the zeros (digit i is slice i + 1);
       // windows at even digits, then at odd ones from the zeros
-      const int col = STACK == 2 ? w & 3 : w;
-      const bool odd = STACK == 2 && w >= 4;
+      const int col = STACK == 2 ? w % (ND / 2) : w;
+      const bool odd = STACK == 2 && w >= ND / 2;
       wa[w] = (uint32_t)((STACK == 2 ? (odd ? 2 * col : 2 * col + 1) : w) * sh.slA) >> 4;
-      wb[w] = (uint32_t)((odd ? kXDigits / 2 : 0) * sh.slB) >> 4;
+      wb[w] = (uint32_t)((odd ? ND / 2 : 0) * sh.slB) >> 4;
       wc[w] = col * NB;
-      wn[w] = x_idesc(NB * ((STACK == 2 ? 4 : 8) - col), 0);
+      wn[w] = x_idesc(NB * ((STACK == 2 ? ND / 2 : ND) - col), 0);
     }
     const uint64_t desc0 = x_desc(x_smem(smem));
-    const uint32_t d_im_part = (uint32_t)sh.partA >> 4, b_im_part = (uint32_t)(kXDigits * sh.slB) >> 4;
+    const uint32_t d_im_part = (uint32_t)sh.partA >> 4, b_im_part = (uint32_t)(ND * sh.slB) >> 4;
     const bool leader = x_elect();
     int st = 0;
     uint32_t ph = 0;
@@ -682,7 +738,7 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
         const uint32_t first = c == 0 ? 0u : 1u;  // the first window covers every column
         if (leader) {
 #pragma unroll
-          for (int w = 0; w < 8; w++) {
+          for (int w = 0; w < ND; w++) {
             const uint64_t are = da + wa[w], aim = are + d_im_part, bre = db + wb[w], bim = bre + b_im_part;
             x_mma(d_re + wc[w], are, bre, wn[w], w == 0 ? first : 1u);
             x_mma(d_im + wc[w], are, bim, wn[w], w == 0 ? first : 1u);
@@ -718,89 +774,61 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
     const bool top = r < S.nAp, mine = r < STACK * S.nAp;
     long long* dst = sums + (top ? r : r - S.nAp + 2 * NB * S.nAp);  // STACK 2: even levels first, then the odd ones
     const uint32_t tw = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    // the entries of this thread are the same in every product: the first ones stay
+    // in registers (row | column << 16, item at q | item at -q << 16)
+    constexpr int kHeld = STACK == 2 ? 6 : 4;
+    int2 held[kHeld];
+#pragma unroll
+    for (int j = 0; j < kHeld; j++) {
+      const int t = tid + j * 32 * kXEpi;
+      held[j] = t < S.n_ent ? __ldg(S.entries + t) : make_int2(0, -1);  // -1: no items
+    }
+    // exponents are read one product ahead
+    const int jx = tid < S.nA ? __ldg(S.expA + tid) : 0, jy = tid < S.nB ? __ldg(S.expB + tid) : 0;
+    int q = q_of(0), nq = x_neg_site(q, L);
+    int ex_next = __ldg(E + (size_t)q * n_jobs + jx), ey_next = __ldg(E + (size_t)nq * n_jobs + jy);
     for (int i = 0; i < n_mine; i++) {
       const int buf = n_buf == 2 ? i & 1 : 0, m = n_buf == 2 ? i >> 1 : i;
-      const int q = q_of(i), nq = x_neg_site(q, L);
-      int* s_ex = xs.ex[i & 1];
-      int* s_ey = xs.ey[i & 1];
-      if (tid < S.nA) s_ex[tid] = __ldg(E + (size_t)q * n_jobs + __ldg(S.expA + tid));
-      if (tid < S.nB) s_ey[tid] = __ldg(E + (size_t)nq * n_jobs + __ldg(S.expB + tid));
+      short* s_ex = xs.ex[i & 1];
+      short* s_ey = xs.ey[i & 1];
+      // |exponent| < 2^11 (kXBad: 2^15 - 1)
+      if (tid < S.nA) s_ex[tid] = (short)min(ex_next, 0x7fff);
+      if (tid < S.nB) s_ey[tid] = (short)min(ey_next, 0x7fff);
+      Ld* pq = reinterpret_cast<Ld*>(P) + (size_t)q * n_items;
+      Ld* pn = reinterpret_cast<Ld*>(P) + (size_t)nq * n_items;
+      const bool self = STACK == 2 && nq == q;  // q = -q has its products from the items at q
+      if (i + 1 < n_mine) {
+        q = q_of(i + 1);
+        nq = x_neg_site(q, L);
+        ex_next = __ldg(E + (size_t)q * n_jobs + jx);
+        ey_next = __ldg(E + (size_t)nq * n_jobs + jy);
+      }
       const bool ok = x_wait(bar_acc + 8 * buf, (uint32_t)(m & 1), spin_limit, abort_flag);
       if (!x_all_epi(ok)) break;  // one verdict for all of them; the sums of the last product are read
       x_fence_after();
       const uint32_t d_re = tw + buf * bufW, d_im = d_re + bufW / 2;
       for (int j0 = 4 * half; has && j0 < S.nB; j0 += 8) {
-        if (STACK == 2) {
-          // level 2 c in the first rows of D, 2 c + 1 in the next
-          uint32_t a[4][4], b[4][4], wide = 0;
-          constexpr long long off = kXMagic * ((1ll << 28) + (1ll << 14) + 1);
+        // a group's level sums: STACK 2, level 2 c of the first rows of D and 2 c + 1
+        // of the next at column block c; STACK 1, level c at column block c
+        constexpr int NC = STACK == 2 ? ND / 2 : ND;
 #pragma unroll
-          for (int c = 0; c < 4; c++) {
-            x_ld4(d_re + c * NB + j0, a[c]);
-            x_ld4(d_im + c * NB + j0, b[c]);
-          }
+        for (int part = 0; part < 2; part++) {
+          uint32_t a[NC][4], wide = 0;
 #pragma unroll
-          for (int c = 0; c < 4; c++) {
-            x_wait_ld(a[c]);
-            x_wait_ld(b[c]);
-          }
-          const int s1 = top ? 14 : 7, s2 = top ? 0 : 7;
-          long long sr[4], si[4];
+          for (int c = 0; c < NC; c++) x_ld4((part ? d_im : d_re) + c * NB + j0, a[c]);
 #pragma unroll
-          for (int j = 0; j < 4; j++) {
-            const unsigned r0 = x_bits(a[0][j], wide), r1 = x_bits(a[1][j], wide), r2 = x_bits(a[2][j], wide);
-            const unsigned i0 = x_bits(b[0][j], wide), i1 = x_bits(b[1][j], wide), i2 = x_bits(b[2][j], wide);
-            const int r3 = (int)(x_bits(a[3][j], wide) - (unsigned)kXMagic);
-            const int i3 = (int)(x_bits(b[3][j], wide) - (unsigned)kXMagic);
-            sr[j] = ((x_mad(r0, 1u << 28, x_mad(r1, 1u << 14, r2)) - off) << s1) + (r3 >> s2);
-            si[j] = ((x_mad(i0, 1u << 28, x_mad(i1, 1u << 14, i2)) - off) << s1) + (i3 >> s2);
-          }
+          for (int c = 0; c < NC; c++) x_wait_ld(a[c]);
+          long long v[4];
+#pragma unroll
+          for (int j = 0; j < 4; j++) v[j] = x_levels(a, j, top, wide);
           if (wide & 0xff800000u) {
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-              sr[j] = x_sum4(x_int(a[0][j]), x_int(a[1][j]), x_int(a[2][j]), x_int(a[3][j]), top);
-              si[j] = x_sum4(x_int(b[0][j]), x_int(b[1][j]), x_int(b[2][j]), x_int(b[3][j]), top);
-            }
+            for (int j = 0; j < 4; j++) v[j] = x_levels_wide(a, j, top);
           }
           __syncwarp();
           if (mine) {
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-              dst[(j0 + j) * S.nAp] = sr[j];
-              dst[(NB + j0 + j) * S.nAp] = si[j];
-            }
-          }
-        } else {
-#pragma unroll
-          for (int part = 0; part < 2; part++) {
-            uint32_t a[8][4], wide = 0;
-            constexpr long long off = kXMagic * ((1ll << 28) + (1ll << 14) + 1);
-#pragma unroll
-            for (int s = 0; s < 8; s++) x_ld4((part ? d_im : d_re) + s * NB + j0, a[s]);
-#pragma unroll
-            for (int s = 0; s < 8; s++) x_wait_ld(a[s]);
-            long long v[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-              const unsigned n0 = x_bits(a[0][j], wide), n1 = x_bits(a[1][j], wide), n2 = x_bits(a[2][j], wide);
-              const unsigned n3 = x_bits(a[3][j], wide), n4 = x_bits(a[4][j], wide), n5 = x_bits(a[5][j], wide);
-              const int n6 = (int)(x_bits(a[6][j], wide) - (unsigned)kXMagic);
-              const int n7 = (int)(x_bits(a[7][j], wide) - (unsigned)kXMagic);
-              const long long ev = x_mad(n0, 1u << 28, x_mad(n2, 1u << 14, n4)) - off;
-              const long long od = x_mad(n1, 1u << 28, x_mad(n3, 1u << 14, n5)) - off;
-              v[j] = (ev << 14) + n6 + (od << 7) + (n7 >> 7);
-            }
-            if (wide & 0xff800000u) {
-#pragma unroll
-              for (int j = 0; j < 4; j++)
-                v[j] = x_sum4(x_int(a[0][j]), x_int(a[2][j]), x_int(a[4][j]), x_int(a[6][j]), true) +
-                       x_sum4(x_int(a[1][j]), x_int(a[3][j]), x_int(a[5][j]), x_int(a[7][j]), false);
-            }
-            __syncwarp();
-            if (mine) {
-#pragma unroll
-              for (int j = 0; j < 4; j++) dst[(part * NB + j0 + j) * S.nAp] = v[j];
-            }
+            for (int j = 0; j < 4; j++) dst[(part * NB + j0 + j) * S.nAp] = v[j];
           }
         }
       }
@@ -808,11 +836,7 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       __syncwarp();
       if (lane == 0) x_arrive(bar_free + 8 * buf);
       asm volatile("bar.sync 1, %0;" ::"n"(32 * kXEpi) : "memory");  // the sums are in place
-      using Out = typename XRaw<T>::load;
-      Out* pq = reinterpret_cast<Out*>(P + (size_t)q * n_items);
-      Out* pn = reinterpret_cast<Out*>(P + (size_t)nq * n_items);
-      for (int t = tid; t < S.n_ent; t += 32 * kXEpi) {
-        const int2 en = __ldg(S.entries + t);  // row | column << 16; item at q | item at -q << 16
+      auto entry = [&](int2 en) {
         const int row = en.x & 0xffff, col = en.x >> 16;
         const long long* p = sums + col * S.nAp + row;
         long long re = p[0], im = p[NB * S.nAp];
@@ -822,12 +846,14 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
         }
         // the sum is (sum of T_A T_B) 2^-56, T = x 2^(55 - e)
         const int ex = s_ex[row], ey = s_ey[col];
-        const Out v = x_value(Out(), re, im, ex == kXBad || ey == kXBad ? kXBad : ex + ey - 54);
+        const Ld v = x_value(Ld(), re, im, ex == 0x7fff || ey == 0x7fff ? kXBad : ex + ey - 54);
         const int item_q = (int)(short)en.y, item_n = en.y >> 16;
         if (item_q >= 0) pq[item_q] = v;
-        // STACK 2: q = -q has its products from the items at q already
-        if (item_n >= 0 && !(STACK == 2 && nq == q)) pn[item_n] = v;
-      }
+        if (item_n >= 0 && !self) pn[item_n] = v;
+      };
+#pragma unroll
+      for (int j = 0; j < kHeld; j++) entry(held[j]);
+      for (int t = tid + kHeld * 32 * kXEpi; t < S.n_ent; t += 32 * kXEpi) entry(__ldg(S.entries + t));
     }
   }
   // every warp has left its loop: accumulators read, stages free
@@ -836,14 +862,22 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
   x_fence_after();
 }
 
-// F: q-major blocks [V][n_out] (16 bytes per complex value); P[V][n_items]; the
-// trace set runs over the pairs qlist[n_pairs], the slice set over every q.
-// err: bit 1 is set when a wait gave up.
+template <typename T, int FORM>
+__device__ __forceinline__ void exact_form(unsigned char* smem, XShared& xs, const void* blk, int L, int n_out,
+                                           const ExactArgs& A, const int* E, const int* qlist, int n_q, void* P,
+                                           long long spin_limit) {
+  if (A.set[FORM].nAp && (int)blockIdx.x < n_q && !*(volatile int*)&xs.abort)
+    exact_set<T, FORM>(smem, xs, blk, L, n_out, A.set[FORM], E, A.n_jobs, qlist, n_q, P, A.n_items, spin_limit);
+}
+
+// blk: q-major blocks [V][n_out]; P[V][n_items]; the trace sets run over the
+// pairs qlist[n_pairs], the slice sets over every q.  err: bit 1 is set when a
+// wait gave up.
 template <typename T>
 __global__ void __launch_bounds__(kXWarps * 32, 1)
-k_contract_exact(const float4* __restrict__ F, int L, int n_out, const ExactDev trace, const ExactDev slice,
-                 const int* __restrict__ E, int n_jobs, const int* __restrict__ qlist, int n_pairs,
-                 float4* __restrict__ P, int n_items, int* __restrict__ err, long long spin_limit) {
+k_contract_exact(const void* __restrict__ blk, int L, int n_out, const ExactArgs A, const int* __restrict__ E,
+                 const int* __restrict__ qlist, int n_pairs, void* __restrict__ P, int* __restrict__ err,
+                 long long spin_limit) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ XShared xs;
   const int tid = threadIdx.x, warp = tid >> 5, V = L * L * L;
@@ -858,62 +892,67 @@ k_contract_exact(const float4* __restrict__ F, int L, int n_out, const ExactDev 
   __syncthreads();
   x_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&xs.tmem);
-  if (trace.nAp && (int)blockIdx.x < n_pairs)
-    exact_set<T, 2>(smem, xs, F, L, n_out, trace, E, n_jobs, qlist, n_pairs, P, n_items, spin_limit);
-  if (slice.nAp && (int)blockIdx.x < V && !*(volatile int*)&xs.abort)
-    exact_set<T, 1>(smem, xs, F, L, n_out, slice, E, n_jobs, nullptr, V, P, n_items, spin_limit);
+  exact_form<T, kExactTrace>(smem, xs, blk, L, n_out, A, E, qlist, n_pairs, P, spin_limit);
+  exact_form<T, kExactSame>(smem, xs, blk, L, n_out, A, E, qlist, n_pairs, P, spin_limit);
+  exact_form<T, kExactSlice>(smem, xs, blk, L, n_out, A, E, nullptr, V, P, spin_limit);
+  exact_form<T, kExactSliceT>(smem, xs, blk, L, n_out, A, E, nullptr, V, P, spin_limit);
   if (tid == 0 && *(volatile int*)&xs.abort) atomicOr(err, 2);
   if (warp == kXEpi)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kXCols) : "memory");
 }
 
-static bool exact_set_ok(const ExactDev& S, int stack) {
+static bool exact_set_ok(const ExactDev& S, int form) {
   if (S.nAp == 0) return true;
+  const int stack = form < kExactSlice ? 2 : 1;
   // a window of 128 rows that starts at the last slices reads past them into
   // the B digits: that stays inside the stage
   return S.nAp % 16 == 0 && S.nBp % 16 == 0 && S.nA <= S.nAp && S.nB <= S.nBp &&
          (stack == 2 ? S.nAp <= kExactMaxBlocks && S.nAp == S.nBp && S.K == 144
-                     : S.nAp <= kExactMaxSliceA && S.nBp <= kExactMaxSliceB && S.K <= 144 && S.K % 2 == 0) &&
+                     : S.nAp <= kExactMaxSliceA && S.nBp <= kExactMaxSliceB && S.K <= 144 && S.K % 4 == 0) &&
          x_shape(stack, S.nAp, S.nBp).n_stages >= 2;
 }
 
 cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const int* jobs, int n_jobs,
                                    int* E, cudaStream_t st) {
-  if (n_q <= 0 || n_jobs <= 0) return cudaSuccess;
-  if (df) k_exact_exponents<dfr><<<(unsigned)n_q, 256, 0, st>>>((const float4*)blk, n_out, jobs, n_jobs, E);
-  else k_exact_exponents<double><<<(unsigned)n_q, 256, 0, st>>>((const float4*)blk, n_out, jobs, n_jobs, E);
+  if (n_q <= 0 || n_jobs <= 0) return cudaErrorInvalidValue;
+  if (df) k_exact_exponents<dfr><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, jobs, n_jobs, E);
+  else k_exact_exponents<double><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, jobs, n_jobs, E);
   return cudaGetLastError();
 }
 
 template <typename T>
-static cudaError_t launch_exact_t(const float4* F, int L, int n_out, const ExactArgs& a, const int* E,
-                                  const int* qlist, int n_pairs, float4* P, int* err, long long spin_limit, int n_sm,
+static cudaError_t launch_exact_t(const void* blk, int L, int n_out, const ExactArgs& a, const int* E,
+                                  const int* qlist, int n_pairs, void* P, int* err, long long spin_limit, int n_sm,
                                   cudaStream_t st) {
   const int V = L * L * L;
   if (a.n_small > 0) {
-    k_exact_small<T><<<V, 256, 0, st>>>(F, L, n_out, a.tasks, a.small, a.n_small, a.n_items, P);
+    k_exact_small<T><<<V, 256, 0, st>>>(blk, L, n_out, a.tasks, a.small, a.n_small, a.n_items, P);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   size_t sm = 0;
-  if (a.trace.nAp) sm = (size_t)x_shape(2, a.trace.nAp, a.trace.nBp).bytes;
-  if (a.slice.nAp) sm = std::max(sm, (size_t)x_shape(1, a.slice.nAp, a.slice.nBp).bytes);
+  int n_q = n_pairs;
+  for (int form = 0; form < kExactSets; form++) {
+    const ExactDev& S = a.set[form];
+    if (!S.nAp) continue;
+    if (!exact_set_ok(S, form)) return cudaErrorInvalidValue;
+    sm = std::max(sm, (size_t)x_shape(form < kExactSlice ? 2 : 1, S.nAp, S.nBp).bytes);
+    if (form >= kExactSlice) n_q = V;
+  }
+  if (!sm) return cudaErrorInvalidValue;
   static int granted[64] = {0};
   const cudaError_t e = ensure_smem(k_contract_exact<T>, sm, granted);
   if (e != cudaSuccess) return e;
-  const int n_q = a.slice.nAp ? V : n_pairs;
-  k_contract_exact<T><<<std::min(n_q, n_sm), kXWarps * 32, sm, st>>>(F, L, n_out, a.trace, a.slice, E, a.n_jobs, qlist,
-                                                                     n_pairs, P, a.n_items, err, spin_limit);
+  k_contract_exact<T><<<std::min(n_q, n_sm), kXWarps * 32, sm, st>>>(blk, L, n_out, a, E, qlist, n_pairs, P, err,
+                                                                     spin_limit);
   return cudaGetLastError();
 }
 
 cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, const ExactArgs& a, const int* E,
                                   const int* qlist, int n_pairs, void* P, int* err, long long spin_limit,
                                   cudaStream_t st) {
-  if (!a.trace.nAp && !a.slice.nAp) return cudaErrorInvalidValue;
   // 32-byte loads: rows and row length even (exact_split.cpp takes no other plan)
-  if (!exact_set_ok(a.trace, 2) || !exact_set_ok(a.slice, 1) || (n_out & 1) || (((uintptr_t)blk) & 31) || !err)
-    return cudaErrorInvalidValue;
+  if ((n_out & 1) || (((uintptr_t)blk) & 31) || !err) return cudaErrorInvalidValue;
   static int n_sm[64] = {0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -923,30 +962,29 @@ cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, co
     e = cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
-  const float4* F = (const float4*)blk;
-  return df ? launch_exact_t<dfr>(F, L, n_out, a, E, qlist, n_pairs, (float4*)P, err, spin_limit, n_sm[dev], st)
-            : launch_exact_t<double>(F, L, n_out, a, E, qlist, n_pairs, (float4*)P, err, spin_limit, n_sm[dev], st);
+  return df ? launch_exact_t<dfr>(blk, L, n_out, a, E, qlist, n_pairs, P, err, spin_limit, n_sm[dev], st)
+            : launch_exact_t<double>(blk, L, n_out, a, E, qlist, n_pairs, P, err, spin_limit, n_sm[dev], st);
 }
 
-size_t exact_wick_smem(int n_items) { return (size_t)kWickQ * n_items * 16; }
+static size_t wick_smem(int n_items, int n_coefs) { return 16 * (size_t)n_items + (((size_t)n_coefs * 8 + 15) & ~(size_t)15); }
+bool exact_wick_fits(int n_items, int n_coefs) { return wick_smem(n_items, n_coefs) <= kMaxSmemPerBlock; }
 
-cudaError_t launch_exact_wick(const void* P, int V, int n_items, const int* cptr, const int* citem,
-                              const double* ccoef, const float2* ccoef_df, int n_outputs, void* ct, bool df,
-                              cudaStream_t st) {
-  const size_t sm = exact_wick_smem(n_items);
+template <typename T, typename C, typename Acc>
+static cudaError_t launch_wick_t(const void* P, int V, const ExactArgs& a, const C* coefs, int n_outputs, void* ct,
+                                 cudaStream_t st) {
+  const size_t sm = wick_smem(a.n_items, a.wick.n_coefs);
   if (sm > kMaxSmemPerBlock) return cudaErrorInvalidValue;
-  static int granted_d[64] = {0}, granted_f[64] = {0};
-  cudaError_t e = df ? ensure_smem(k_exact_wick<dfr, float2>, sm, granted_f)
-                     : ensure_smem(k_exact_wick<double, double>, sm, granted_d);
+  static int granted[64] = {0};
+  const cudaError_t e = ensure_smem(k_exact_wick<T, C, Acc>, sm, granted);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((V + kWickQ - 1) / kWickQ);
-  if (df)
-    k_exact_wick<dfr, float2><<<grid, kWickThreads, sm, st>>>((const float4*)P, V, n_items, cptr, citem, ccoef_df, n_outputs,
-                                                     (float4*)ct);
-  else
-    k_exact_wick<double, double><<<grid, kWickThreads, sm, st>>>((const float4*)P, V, n_items, cptr, citem, ccoef, n_outputs,
-                                                        (float4*)ct);
+  k_exact_wick<T, C, Acc><<<(unsigned)V, kWickThreads, sm, st>>>(P, a.n_items, a.wick, coefs, n_outputs, ct);
   return cudaGetLastError();
+}
+
+cudaError_t launch_exact_wick(const void* P, int V, const ExactArgs& a, bool df, int n_outputs, void* ct,
+                              cudaStream_t st) {
+  return df ? launch_wick_t<dfr, float2, WickAccDf>(P, V, a, a.wick.coefs_df, n_outputs, ct, st)
+            : launch_wick_t<double, double, WickAcc64>(P, V, a, a.wick.coefs, n_outputs, ct, st);
 }
 
 }  // namespace bbc

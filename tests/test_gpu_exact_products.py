@@ -1,6 +1,7 @@
 """GPU tests of the digit-sliced tensor-core products of the FP64-accurate
 paths: operand counts that leave ragged tiles (one channel: 12 blocks, a few,
-all 64 octet ids: 48 blocks), small lattices (fewer pairs than SMs, q = -q
+all 64 octet ids: 48 blocks; decuplet ids: same-orientation traces and
+transposed slices), small lattices (fewer pairs than SMs, q = -q
 only), rows of very different size, zero and non-finite propagators.
 
 Tolerance: the 1e-12 of the FP64-accurate paths (relative to the channel's
@@ -46,7 +47,8 @@ def _check(got, want, vanish=()):
 
 @pytest.mark.parametrize("precision", [0, 3])
 @pytest.mark.parametrize("L,chans,lower", [(2, [0], False), (2, list(range(64)), False), (4, [1, 2], True),
-                                           (4, [11, 20, 51], False), (4, list(range(52)), False)])
+                                           (4, [11, 20, 51], False), (4, list(range(52)), False),
+                                           (4, [64, 70, 99, 143, 145, 150], False), (2, list(range(145, 154)), True)])
 def test_operand_counts(bbc, precision, L, chans, lower):
     F = synth.flavour_set(L, 4, 0, 0.3, 0.4, seed=90 + L, times=[0])
     want = orc.correlator(L, F["u"][0], F["u"][0], F["s"][0], chans, lower=lower)
