@@ -72,7 +72,9 @@ typedef enum {
 } bbc_status;
 
 typedef enum {
-  BBC_FP64 = 0,      /* blocks, FFTs, contraction and sums in FP64 */
+  BBC_FP64 = 0,      /* blocks, FFTs, contraction and sums in FP64; the block-pair
+                         products as exact products of 7-bit digits of 55-bit fixed-point
+                         values on the tensor cores where the plan allows */
   BBC_MIXED_FP32 = 1, /* blocks, FFTs and block-pair products in FP32 after an exact
                          per-slice power-of-two rescaling of each propagator; the signed
                          sum over Wick diagrams in double-float arithmetic (two FP32
@@ -96,8 +98,9 @@ typedef enum {
                          only (EINVAL at creation for channel lists that do not fit it) */
   BBC_DF64 = 3,       /* FP64-accurate results from double-float arithmetic
                          (unevaluated sums of two FP32 values, 48-bit significand) on
-                         the FP32 pipes: propagators, blocks, FFTs, block-pair products
-                         and Wick sums; FP64 only to split the input and to normalise */
+                         the FP32 pipes: propagators, blocks, FFTs and Wick sums; the
+                         block-pair products as for BBC_FP64; FP64 only to split the
+                         input and to normalise */
   BBC_MIXED_TF32 = 4  /* trial: as BBC_MIXED_FP32, with the tensor-core operands rounded
                          once to TF32 (10-bit mantissa, round to nearest) instead of
                          split into two TF32 words: a third of the tensor-core work at
@@ -319,15 +322,17 @@ bbc_status bbc_check_bounded_wait(bbc_ctx* ctx, long long spin_limit);
  *  fused_steps: open-index steps whose rows a lane loads before multiplying
  *    (1; or 2 with 8 or 12 warps, which leave the registers for it);
  *  pair_groups (BBC_FP64, BBC_DF64 and the unfused FP32 route): warp task
- *    lists of the block-pair products per 32 q (48, 96, 192 or 384); more,
- *    shorter lists shorten the tail of the launch;
+ *    lists of the CUDA-core block-pair products per 32 q (48, 96, 192 or 384);
+ *    more, shorter lists shorten the tail of the launch (no effect where the
+ *    products run on the tensor cores);
  *  tc_kernel (mixed FP32 / TF32 with tensor cores): 0 = the trace-form
  *    products on tcgen05 (one persistent CTA per SM, then the CUDA-core
  *    kernel), 1 = on mma.sync, with the CUDA-core kernel of one quarter of
  *    the pairs beside the tensor-core kernel of the next on a second stream
  *    from 4096 pairs {q, -q} on.
  * A new context starts with (1, 256, 16, 18, 1, 48, 0) (pair_groups 192 for
- * BBC_DF64), or with the configuration bbc_autotune chose earlier in the
+ * BBC_DF64; 512 build threads for BBC_FP64 and BBC_DF64 where two build CTAs
+ * fill an SM's shared memory), or with the configuration bbc_autotune chose earlier in the
  * process for the same L, precision and channel list. */
 typedef struct {
   int build_sites, build_threads;

@@ -464,6 +464,17 @@ bbc_status bbc_create_components(bbc_ctx** ctx, const bbc_lattice* lat, bbc_prec
     }
     c->exact = c->ex.all && bbc::exact_wick_fits(16 * (int)c->plan.tasks.size(), (int)c->ex.wick_coefs.size());
   }
+  // Block build of the FP64-accurate precisions: where shared memory holds at
+  // most two one-site CTAs per SM (two octet diquarks and 4548 tensor entries: 89 KB),
+  // 512 threads instead of 256 double the warps that hide its latency.  Per 16^3
+  // slice, 256 against 512 threads: 52 channels FP64 1879 and 1699 us,
+  // double-float 724 and 583; Lambda N 1473 and 1336, 559 and 444.  Plans of smaller
+  // CTAs fill the SM either way and pay for the wider barriers: N N (36 KB, six CTAs)
+  // 426 and 432, 116 and 134; decuplet ids 64..153 (51 KB, four) 1589 and 1632, 445 and 494.
+  constexpr size_t kSmemPerSm = 228 * 1024, kSmemReserved = 1024;
+  if (fp64_storage(prec) &&
+      kSmemPerSm / (bbc::block_build_smem(c->plan.z_slots, 1, true, (int)c->plan.diquarks.size()) + kSmemReserved) <= 2)
+    c->tune.build_threads = 512;
   // warp task groups of the pair products: enough warps per 32 q to fill the
   // GPU several times over at L = 16 (V/32 q tiles x groups warps); the
   // double-float products start with more, shorter groups (fewer q tiles in
