@@ -41,9 +41,6 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 #: 8 flops each: a complex product takes at least three real multiplications
 #: (Gauss), so at most 629 G FMA/s / 3 = 209.8 G complex MACs/s = 1.678 TFLOP/s
 FP64_CMAC_PEAK_TFLOPS = FP64_PEAK_TFLOPS * 8.0 / 6.0
-CMAC_PEAK_SOURCE = ("derived: 152 SM x 2 FP64 FMA/clk x 2070 MHz = 629.3 G FMA/s; a complex multiply-add (8 "
-                    "algorithmic flops) needs at least 3 real FMAs (three-multiplication complex product), so the "
-                    "FP64 pipe's ceiling is 209.8 G complex MACs/s = 1.678 TFLOP/s")
 #: FP32 FMA peak: 152 SMs x 128 lanes x 2 flop x 2070 MHz (probe: 74.8 TFLOP/s)
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
@@ -62,6 +59,27 @@ def measured_hbm_gbs(path=os.path.join(os.path.dirname(os.path.abspath(__file__)
 
 
 HBM_PEAK_GBS, HBM_PEAK_SOURCE = measured_hbm_gbs()
+
+
+def measured_bf16_tflops(path=os.path.join(os.path.dirname(os.path.abspath(__file__)), "MEASURED_PEAKS.json")):
+    """cuBLAS bf16 burst rate (TFLOP/s) from the peaks file; 1900 without it."""
+    try:
+        v = float(json.load(open(path))["bf16_tflops"])
+        if v > 0:
+            return v
+    except (OSError, ValueError, KeyError, TypeError):
+        pass
+    return 1900.0
+
+
+#: the FP64-accurate block-pair products run as exact products of 7-bit digits
+#: in fp16 on the tensor cores: 36 digit pairs per complex multiply-add, four
+#: real products each, so the fp16 rate gives this many algorithmic TFLOP/s (8
+#: flops per complex multiply-add)
+DIGIT_PAIRS = 36
+DIGIT_CMAC_PEAK_TFLOPS = measured_bf16_tflops() / DIGIT_PAIRS
+DIGIT_PEAK_SOURCE = ("derived: measured cuBLAS bf16 burst rate / 36 digit pairs per complex multiply-add (four real "
+                     "16-bit products each; 8 algorithmic flops per complex multiply-add)")
 
 
 def profiled_traffic(path, kernel_src, pair_items):
@@ -427,21 +445,17 @@ def run_ours(args, torch, rank, world, local):
     value = shard.job_throughput(V * T * N_CH, world, ms)
     value_e2e = shard.job_throughput(V * T * N_CH, world, ms_e2e)
 
-    # dominant kernel: the contraction (FP64 ALU bound)
+    # the contraction (its stage: the digit-sliced tensor-core products and the small tasks)
     c_ms, c_n = stages["contract"]
     c_avg_ms = c_ms / max(c_n, 1)
     flops_per_launch = 8.0 * sizes["pair_macs_per_site"] * V
     achieved = flops_per_launch / (c_avg_ms * 1e-3) / 1e12
-    here = os.path.dirname(os.path.abspath(__file__))
-    traffic = profiled_traffic(os.path.join(here, "profiles", "k_pair_products_f64_L16_slice.md"),
-                               os.path.join(here, "paper_1510_00903_gb300", "csrc", "pair_products.cu"),
-                               sizes["pair_items"])
-    roofline = {"bound": "alu", "kernel": "k_pair_products<double>", "achieved": achieved,
-                "peak": FP64_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_CMAC_PEAK_TFLOPS,
-                "traffic": traffic, "peak_source": CMAC_PEAK_SOURCE,
+    roofline = {"bound": "tensor", "kernel": "k_contract_exact<double>", "achieved": achieved,
+                "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / DIGIT_CMAC_PEAK_TFLOPS,
+                "traffic": None, "peak_source": DIGIT_PEAK_SOURCE,
                 "algorithmic_flop_per_launch": flops_per_launch, "avg_launch_ms": c_avg_ms}
     stage_ms = {k: v[0] / args.steps for k, v in stages.items()}
-    step_roof = step_roofline(counts, V, T, stage_ms, ms)
+    step_roof = step_roofline(counts, V, T, stage_ms, ms, cmac_tflops=DIGIT_CMAC_PEAK_TFLOPS)
 
     def mixed_leg(precision, note, components=bbc.BBC_UPPER):
         corm = bbc.Correlators(L, T, 0, M_UD, M_S, channels=chans, precision=precision, device=dev, stream=stream,
@@ -725,10 +739,10 @@ def run_decuplet(args, torch, dev, bbc, synth):
                      "L": L, "T": T, "channels": len(chans),
                      "l2": f"no flush: block fields of one slice ({V * sizes['block_outputs'] * 16 / 1e6:.0f} MB) "
                            "exceed the 129 MB L2"},
-          "roofline": {"bound": "alu", "kernel": "k_pair_products<double>", "achieved": fp["contract_tflops"],
-                       "peak": FP64_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s",
-                       "frac": fp["contract_tflops"] / FP64_CMAC_PEAK_TFLOPS, "traffic": None,
-                       "peak_source": CMAC_PEAK_SOURCE},
+          "roofline": {"bound": "tensor", "kernel": "k_contract_exact<double>", "achieved": fp["contract_tflops"],
+                       "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s",
+                       "frac": fp["contract_tflops"] / DIGIT_CMAC_PEAK_TFLOPS, "traffic": None,
+                       "peak_source": DIGIT_PEAK_SOURCE},
           "plan": sizes, "fp64": fp, "df64": legs["df64"], "mixed": legs["mixed"], "clocks": clocks})
 
 
@@ -797,17 +811,6 @@ L5, T5, N_SRC5 = 48, 96, 4
 #: slices per headline step: a quarter of one source's time slices, so 16
 #: steps cover the four sources once and 20 timed steps stay near a minute
 HEAD_SLICES = 24
-#: double-float arithmetic on the FP32 pipes: one complex multiply-add of the
-#: block-pair products is four double-float multiply-adds of 12 FP32
-#: instructions each (TwoProduct of the high words, the cross terms, TwoSum
-#: into the accumulator)
-DF_INSTR_PER_CMAC = 48
-#: FP32 instruction issue of the whole GPU: 152 SMs x 128 lanes x 2070 MHz
-FP32_ISSUE_TOPS = 152 * 128 * 2.070e9 / 1e12
-DF_CMAC_PEAK_TFLOPS = FP32_ISSUE_TOPS / DF_INSTR_PER_CMAC * 8.0
-DF_PEAK_SOURCE = "derived: 40.27 T FP32 instr/s / 48 instr per double-float complex MAC x 8 flop"
-
-
 def channel_errors(torch, got, ref):
     """Per channel: max over r and spin of |got - ref| / max |ref| (device tensors [n_ch, V, 16]);
     returns the maximum and median over channels and the worst channel."""
@@ -866,7 +869,6 @@ def run_default(args, torch, dev, bbc, synth):
     rank, world, local = dist_env()
     chans = list(range(N_CH))
     V5 = L5 ** 3
-    here = os.path.dirname(os.path.abspath(__file__))
     stream = torch.cuda.Stream(dev)
     # one source's wall-source propagators (complex64); the four sources share the draw
     S_dev = [device_propagators(torch, dev, L5, T5, 0, m, 1000 * rank + s) for m, s in ((M_UD, 91), (M_S, 92))]
@@ -908,12 +910,6 @@ def run_default(args, torch, dev, bbc, synth):
     c_avg = stage_tot["contract"] / max(n_contract, 1)
     flop = 8.0 * sizes["pair_macs_per_site"] * V5
     achieved = flop / (c_avg * 1e-3) / 1e12
-    # DRAM bytes per launch from the ncu capture of the 16^3 slice (the full-size
-    # launch is too large to capture), scaled to 48^3 by the sites processed
-    traffic16 = profiled_traffic(os.path.join(here, "profiles", "k_pair_products_df_L16_slice.md"),
-                                 os.path.join(here, "paper_1510_00903_gb300", "csrc", "pair_products_df.cu"),
-                                 sizes["pair_items"])
-    traffic = None if traffic16 is None else traffic16 * V5 / L_BENCH ** 3
     value = shard.job_throughput(HEAD_SLICES * V5 * N_CH, world, ms)
     # e2e: pinned host propagators in, pinned host correlators out (two-slice ring)
     S_host = [x[:HEAD_SLICES].cpu().pin_memory() for x in S_dev]
@@ -999,16 +995,14 @@ def run_default(args, torch, dev, bbc, synth):
             ref16 = out2[16].clone()
             ca = st16["contract"][0] / max(st16["contract"][1], 1)
             ach = 8.0 * sz["pair_macs_per_site"] * V2 / (ca * 1e-3) / 1e12
-            leg["roofline"] = {"kernel": "k_pair_products<double>", "achieved": round(ach, 4),
-                               "peak": FP64_CMAC_PEAK_TFLOPS, "frac": round(ach / FP64_CMAC_PEAK_TFLOPS, 4),
-                               "traffic": profiled_traffic(
-                                   os.path.join(here, "profiles", "k_pair_products_f64_L16_slice.md"),
-                                   os.path.join(here, "paper_1510_00903_gb300", "csrc", "pair_products.cu"),
-                                   sz["pair_items"])}
+            leg["roofline"] = {"kernel": "k_contract_exact<double>", "achieved": round(ach, 4),
+                               "peak": DIGIT_CMAC_PEAK_TFLOPS, "frac": round(ach / DIGIT_CMAC_PEAK_TFLOPS, 4),
+                               "traffic": None}
         else:
             leg["err_vs_fp64"] = channel_errors(torch, out2[16], ref16)
         if prec in (bbc.BBC_FP64, bbc.BBC_MIXED_FP32):
-            roof = step_roofline(cnt, V2, T2_, sm16, m16, mixed=prec == bbc.BBC_MIXED_FP32)
+            roof = step_roofline(cnt, V2, T2_, sm16, m16, mixed=prec == bbc.BBC_MIXED_FP32,
+                                 cmac_tflops=DIGIT_CMAC_PEAK_TFLOPS)
             leg["step_roofline"] = {"floor_ms": round(roof["floor_ms"], 3), "frac": round(roof["frac"], 4)}
             leg["stage_ms"] = {k: round(v, 2) for k, v in sm16.items() if v}
         if name == "fp64":
@@ -1047,9 +1041,9 @@ def run_default(args, torch, dev, bbc, synth):
                 "h2d_bytes_per_step": int(HEAD_SLICES * 2 * V5 * 144 * 8),
                 "d2h_bytes_per_step": int(HEAD_SLICES * N_CH * V5 * 16 * 16)},
         "gpu_launches": launches,
-        "roofline": {"bound": "alu", "kernel": "k_pair_products_df", "achieved": achieved, "peak": DF_CMAC_PEAK_TFLOPS,
-                     "unit": "TFLOP/s", "frac": achieved / DF_CMAC_PEAK_TFLOPS, "traffic": traffic,
-                     "peak_source": DF_PEAK_SOURCE, "avg_launch_ms": round(c_avg, 3)},
+        "roofline": {"bound": "tensor", "kernel": "k_contract_exact<dfr>", "achieved": achieved,
+                     "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / DIGIT_CMAC_PEAK_TFLOPS,
+                     "traffic": None, "peak_source": DIGIT_PEAK_SOURCE, "avg_launch_ms": round(c_avg, 3)},
         "err_vs_fp64": head_err,
         "stage_ms_per_step": {k: round(v, 1) for k, v in stage_ms.items() if v > 0.5},
         # legs, one array each: [site*channels/s, ms per step, step roofline frac, max per-channel error vs FP64]
