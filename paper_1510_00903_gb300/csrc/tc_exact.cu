@@ -17,9 +17,10 @@
 // A digit pair costs 4 real MACs per complex one at 4096 MACs per clock and
 // SM against 2 FP64 FMAs per clock (three per complex MAC) or 128 FP32 lanes
 // (48 instructions per complex MAC in double-float): 36 digit pairs are still
-// many times cheaper than either pipe.  What bounds the kernel is the tensor
-// pipe together with the integer work of making the digits (about 35
-// instructions per real value).  Measured against the CUDA-core products of
+// many times cheaper than either pipe.  What bounds the kernel is the integer
+// work of making the digits (about 35 instructions per real value) beside the
+// tensor pipe, and the drain of the one accumulator set: 50% of the issue slots,
+// 37% of the tensor pipe, 22% of DRAM at 16^3.  Measured against the CUDA-core products of
 // field-major blocks, 52 channels: FP64 16^3 3.99 -> 0.57 ms per slice,
 // double-float 16^3 1.40 -> 0.52, 48^3 35.2 -> 13.0 (both with the small tasks).
 // On field-major blocks (16-byte loads 64 KB and more apart) the same kernel was
