@@ -76,12 +76,14 @@ __device__ __forceinline__ void df_renorm(df64acc& acc) {
 // error word, a product the TwoProduct of the high words with the cross
 // terms added into its error word, and neither renormalises (hi, lo) so that
 // |lo| <= ulp(hi) / 2.  The low word then holds the accumulated rounding
-// errors of a few operations at most a few ulps of the high word; every
+// errors of a few operations, a few ulps of their operands: of the high word
+// too unless the high words cancelled, when it may be as large.  Every
 // later TwoSum and TwoProduct on the high words is still exact, so the error
 // of a sum or product stays about 2^-44 (|a| + |b|) or 2^-44 |a b|: an
 // absolute error at the scale of the operands, which is what the correlator
 // tolerance measures.  Consumers read hi + lo (the pair products, the
-// conversion to double), never hi alone.
+// conversion to double), never hi alone; who needs |lo| <= ulp(hi) / 2
+// normalises first (the last forward FFT pass does for the digit-sliced products).
 struct dfr {
   float hi, lo;
   __host__ __device__ dfr() {}

@@ -185,6 +185,23 @@ __device__ __forceinline__ void line_base(int N, int axis, int line, int& base, 
 // sums the three-multiplication complex products of the contraction read).
 enum { FFT_SITE2FIELD = 0, FFT_FIELD = 1, FFT_FIELD2OUT = 2, FFT_SITE = 3, FFT_SITE2OUT = 4, FFT_FIELD_SUM = 5 };
 
+// A value as its pass stores it.  The last forward pass of the q-major layout
+// (z axis) leaves double-float pairs normalised, hi = RN(hi + lo) and lo the exact
+// rest: the operators do not, and where the high words of a smooth field cancel at
+// q != 0 the low word may be as large as the value, while the digit-sliced products
+// (tc_exact.cu) read a low word of at most half an ulp of the high one.  One TwoSum
+// per real value, free in a pass that HBM bounds.
+template <int MODE, bool INV, typename O>
+__device__ __forceinline__ cpx<O> fft_stored(cpx<O> v, int axis) {
+  if constexpr (std::is_same<O, dfr>::value && MODE == FFT_SITE && !INV) {
+    if (axis == 2) {
+      two_sum(v.re.hi, v.re.lo, v.re.hi, v.re.lo);
+      two_sum(v.im.hi, v.im.lo, v.im.hi, v.im.lo);
+    }
+  }
+  return v;
+}
+
 // S: storage of the input (and of the output in the in-place modes), R:
 // compute type, O: storage of the output of the last inverse pass.
 template <typename S, typename R, int N, bool INV, int MODE, typename O = S>
@@ -243,7 +260,7 @@ k_fft(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned total, i
   } else if (MODE == FFT_SITE) {
     cpx<O>* p = out + (o * V + base) * n_inner + inner;
 #pragma unroll
-    for (int k = 0; k < N; k++) p[(long long)k * stride * n_inner] = cpx<O>(v[k]);
+    for (int k = 0; k < N; k++) p[(long long)k * stride * n_inner] = fft_stored<MODE, INV>(cpx<O>(v[k]), axis);
   } else if (MODE == FFT_SITE2OUT) {
     // inner = channel * 16 + spin; out[ch][r][16].  The scale (1/V, the
     // undone propagator rescaling, the mass factor) may lie far outside the
@@ -270,8 +287,13 @@ k_fft(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned total, i
 // radix-3 butterfly into X[k2], X[k2 + M], X[k2 + 2M] and stores them.  The
 // modes, index decomposition and output forms are those of k_fft.
 constexpr int kSplitLines = 64;  // lines per CTA of 3 x 64 threads
+// Four CTAs per SM fill the shared memory; the double-float q-major pass, which
+// also normalises its pairs, is held to their registers (with three CTAs a 48^3
+// slice's transform took 2.8 ms more).
+template <typename R, int MODE>
+constexpr int split_ctas() { return std::is_same<R, dfr>::value && MODE == FFT_SITE ? 4 : 0; }
 template <typename S, typename R, int M, bool INV, int MODE, typename O = S>
-__global__ void __launch_bounds__(3 * kSplitLines)
+__global__ void __launch_bounds__(3 * kSplitLines, split_ctas<R, MODE>())
 k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned total, int n_inner, int axis,
             const double* __restrict__ scale, O* __restrict__ sum) {
   constexpr int N = 3 * M;
@@ -385,7 +407,7 @@ k_fft3split(const cpx<S>* __restrict__ in, cpx<O>* __restrict__ out, unsigned to
       if (MODE == FFT_FIELD) {
         out[o * V + base + (long long)k * stride] = cpx<O>(x[c]);
       } else if (MODE == FFT_SITE) {
-        out[(o * V + base + (long long)k * stride) * n_inner + inner] = cpx<O>(x[c]);
+        out[(o * V + base + (long long)k * stride) * n_inner + inner] = fft_stored<MODE, INV>(cpx<O>(x[c]), axis);
       } else if (MODE == FFT_SITE2OUT) {  // inner = channel * 16 + spin
         const O f = (O)scale[inner >> 4];
         out[((long long)(inner >> 4) * V + base + (long long)k * stride) * 16 + (inner & 15)] =

@@ -171,9 +171,11 @@ __device__ __forceinline__ unsigned long long x_fix(double x, int e) {
 }
 // Double-float values by rounding FP32 additions (x + M keeps the nearest
 // integer of |x| < 2^22 in its low bits; the residues are exact): 21 bits and
-// 17 bits of the high word, then the rest of it with the low word (the low word
-// is a few units of the high word's last place, so their sum loses nothing that
-// T holds), 17 + 17 bits.  FP32 additions run at twice the rate of shifts.
+// 17 bits of the high word, then the rest of it with the low word, 17 + 17 bits.
+// The pairs are normalised (the forward transform's last pass): |lo| <= 2^-24 |hi|,
+// so that lo 2^(38 - e) stays below 2^14 beside a rest of at most 2^16.  An
+// unnormalised low word could leave the range of x + M and give wrong digits.
+// FP32 additions run at twice the rate of shifts.
 __device__ __forceinline__ unsigned long long x_fix(dfr x, int e) {
   const float M = 12582912.f, p17 = 131072.f;  // 1.5 2^23, 2^17
   const float s = __int_as_float((127 + 21 - e) << 23);  // 2^(21 - e), e >= -72
