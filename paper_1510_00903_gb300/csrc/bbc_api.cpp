@@ -840,7 +840,7 @@ bbc_status bbc_build_blocks(bbc_ctx* c, int n_slots) {
     if (e != cudaSuccess) return cuda_fail(c, e, "forward FFT");
     if (c->exact) {
       e = bbc::launch_exact_exponents(c->d_blk, c->prec == BBC_DF64, (long long)n_slots * c->V, p.n_out,
-                                      c->ex_args.jobs, c->ex_args.n_jobs, c->d_exE, c->stream);
+                                      c->ex_args, c->d_exE, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "row exponents");
     }
     if (c->prec == BBC_MIXED_BF16) {

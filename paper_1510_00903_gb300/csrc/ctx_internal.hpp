@@ -191,7 +191,7 @@ inline void row_terms(const Plan& p, bool fp64, bool powers, std::vector<int2>* 
 }
 
 // Device tables of the digit-sliced contraction, packed into one array of ints:
-// jobs and small tasks, the Wick sums, then per set rowA, rowB, expA, expB and the needed entries (padded to 16
+// exponent pieces and jobs, small tasks, the Wick sums, then per set rowA, rowB, expA, expB and the needed entries (padded to 16
 // bytes); *a points into it at `base`.
 inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, ExactArgs* a) {
   std::vector<int> t;
@@ -203,7 +203,9 @@ inline std::vector<int> exact_tables(const ExactSplit& s, const int* base, Exact
   };
   a->n_jobs = (int)s.jobs.size() / 2;
   a->n_small = (int)s.small.size();
-  a->jobs = put(s.jobs.data(), sizeof(int) * s.jobs.size());
+  a->n_loads = (int)s.loads.size() / 4;
+  a->loads = (const int4*)put(s.loads.data(), sizeof(int) * s.loads.size());
+  a->jobs = (const int2*)put(s.jobs.data(), sizeof(int) * s.jobs.size());
   a->small = put(s.small.data(), sizeof(int) * s.small.size());
   WickDev& w = a->wick;
   w.n_chunks = (int)s.wick_chunks.size();

@@ -128,50 +128,56 @@ void make_exact_split(const Plan& plan, ExactSplit* out) {
     trace_set(plan, f, &S.set[kExactTrace + f], &done);
     slice_set(plan, f, &S.set[kExactSlice + f], &done);
   }
-  // exponent jobs (first row, rows): one per trace block, and one per slice that
-  // lies in no trace block (a slice inside one shares its exponent)
-  std::map<std::pair<int, int>, int> job_of;
-  auto job = [&](int first, int rows) {
-    auto it = job_of.find({first, rows});
-    if (it != job_of.end()) return it->second;
-    const int id = (int)(S.jobs.size() / 2);
-    S.jobs.push_back(first);
-    S.jobs.push_back(rows);
-    job_of[{first, rows}] = id;
-    return id;
-  };
-  std::set<int> blocks;
+  // One exponent per operand row (first field row, rows or kExactColumns).  A slice
+  // inside a trace block has its own: it is one Dirac component of an open index and
+  // may be orders of magnitude smaller than the rest of the block.  Its rows are read
+  // once, with the block's.
+  using Job = std::pair<int, int>;
+  std::map<Job, int> job_of;
+  auto span = [](const Job& j) { return j.second == kExactColumns ? 11 * 12 + 3 : j.second; };
+  for (int f = 0; f < 2; f++) {
+    for (int r : S.set[f].rowA) job_of[{r, 144}] = 0;
+    for (int r : S.set[kExactSlice + f].rowA) job_of[{r, f == 0 ? 36 : kExactColumns}] = 0;
+    for (int r : S.set[kExactSlice + f].rowB) job_of[{r, 36}] = 0;
+  }
+  if (job_of.empty()) return;
+  std::map<Job, std::vector<Job>> loads;
+  for (const auto& j : job_of)
+    if (j.first.second == 144) loads[j.first].push_back(j.first);
+  for (const auto& j : job_of) {
+    if (j.first.second == 144) continue;
+    auto it = loads.upper_bound({j.first.first, 144});
+    const bool inside = it != loads.begin() && j.first.first + span(j.first) <= span(std::prev(it)->first) + std::prev(it)->first.first;
+    loads[inside ? std::prev(it)->first : Job(j.first.first, span(j.first))].push_back(j.first);
+  }
   bool ok = plan.n_out % align == 0;
+  for (const auto& l : loads) {
+    const int id = (int)S.jobs.size() / 2, first = l.first.first;
+    S.loads.insert(S.loads.end(), {first, l.first.second, id, id + (int)l.second.size()});
+    // every operand row lies inside the block rows
+    ok &= first >= 0 && first + l.first.second <= plan.n_out;
+    for (const Job& j : l.second) {
+      job_of[j] = (int)S.jobs.size() / 2;
+      S.jobs.insert(S.jobs.end(), {j.first - first, j.second});
+    }
+  }
   for (int f = 0; f < 2; f++) {
     ExactSet& T = S.set[f];
     for (int r : T.rowA) {
-      blocks.insert(r);
-      T.expA.push_back(job(r, 144));
+      T.expA.push_back(job_of[{r, 144}]);
       ok &= r % align == 0;
     }
     T.expB = T.expA;
-  }
-  auto slice_job = [&](int r, int len) {
-    auto it = blocks.upper_bound(r);
-    if (it != blocks.begin() && r + len <= *std::prev(it) + 144) return job(*std::prev(it), 144);
-    return job(r, len);
-  };
-  for (int f = 0; f < 2; f++) {
     ExactSet& C = S.set[kExactSlice + f];
-    // rows an operand spans: 36, or 11 x 12 + 3 for three columns of a block
-    const int lenA = f == 0 ? 36 : 135;
     for (int r : C.rowA) {
-      C.expA.push_back(slice_job(r, lenA));
+      C.expA.push_back(job_of[{r, f == 0 ? 36 : kExactColumns}]);
       ok &= f == 1 || r % align == 0;
     }
     for (int r : C.rowB) {
-      C.expB.push_back(slice_job(r, 36));
+      C.expB.push_back(job_of[{r, 36}]);
       ok &= r % align == 0;
     }
   }
-  if (S.jobs.empty()) return;
-  // every operand row lies inside the block rows
-  for (size_t j = 0; j < S.jobs.size(); j += 2) ok &= S.jobs[j] >= 0 && S.jobs[j] + S.jobs[j + 1] <= plan.n_out;
   for (int ti = 0; ti < n; ti++) {
     const PairTask& t = plan.tasks[ti];
     if (done[ti]) continue;

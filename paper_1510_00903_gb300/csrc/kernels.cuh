@@ -219,6 +219,7 @@ constexpr int kExactMaxSliceA = 128;  // rows of one instruction
 constexpr int kExactMaxSliceB = 32;
 constexpr int kExactSmallSteps = 16;  // open indices of a small task
 constexpr int kExactSets = 4;
+constexpr int kExactColumns = -36;    // "rows" of an exponent job over three columns of a 12 x 12 block
 // forms of a set: trace tr(M_A M_B), the same without the transpose, slices of
 // 36 consecutive rows, slices whose A side is three columns of a block
 enum { kExactTrace = 0, kExactSame = 1, kExactSlice = 2, kExactSliceT = 3 };
@@ -239,12 +240,14 @@ struct WickDev {  // signed sums: outputs sorted by length, 32 per chunk, lane-i
 struct ExactArgs {
   ExactDev set[kExactSets];  // by form
   WickDev wick;
-  int n_jobs, n_small, n_items;
-  const int *jobs, *small;  // (first row, rows) per exponent job; task ids
+  int n_loads, n_jobs, n_small, n_items;
+  const int4* loads;  // ExactSplit::loads
+  const int2* jobs;   // ExactSplit::jobs
+  const int* small;   // task ids
   const DevTask* tasks;
 };
-cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const int* jobs, int n_jobs,
-                                   int* E, cudaStream_t st);
+cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const ExactArgs& a, int* E,
+                                   cudaStream_t st);
 cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, const ExactArgs& a, const int* E,
                                   const int* qlist, int n_pairs, void* P, int* err, long long spin_limit,
                                   cudaStream_t st);

@@ -211,7 +211,9 @@ struct ExactSet {
 };
 struct ExactSplit {
   ExactSet set[4];                     // by form: kExactTrace .. kExactSliceT (kernels.cuh)
-  std::vector<int> jobs;               // (first field row, rows) per exponent job
+  // row exponents: pieces of rows read once (first field row, rows, first job, last
+  // job + 1), and per job (row in its piece, rows or kExactColumns)
+  std::vector<int> loads, jobs;
   std::vector<int> small;              // tasks with few open indices, one product per thread
   bool all = false;                    // the sets and `small` make every product of the plan
   // signed sums over Wick diagrams: outputs sorted by length, 32 per chunk, entry k

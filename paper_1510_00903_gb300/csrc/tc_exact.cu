@@ -382,8 +382,8 @@ __host__ __device__ inline XShape x_shape(int stack, int nAp, int nBp) {
 }  // namespace
 
 // Exponents of one q per CTA: E[q][job] with max |component| over the job's
-// rows below 0.985 2^E (kXBad: a NaN or infinite value among them); a warp per
-// job, one pass over the operand rows: HBM bound.
+// rows below 0.985 2^E (kXBad: a NaN or infinite value among them).  A warp takes a
+// piece of rows (a whole block) and, from the same loads, the jobs inside it: HBM bound.
 __device__ __forceinline__ int x_mag(const double2& v) {  // the exponent-carrying words
   return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
 }
@@ -392,23 +392,33 @@ __device__ __forceinline__ int x_mag(const float4& v) {  // both words of a doub
 }
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_exact_exponents(const void* __restrict__ blk, int n_out, const int* __restrict__ jobs, int n_jobs,
-                  int* __restrict__ E) {
+k_exact_exponents(const void* __restrict__ blk, int n_out, const int4* __restrict__ loads, int n_loads,
+                  const int2* __restrict__ jobs, int n_jobs, int* __restrict__ E) {
   using Ld = typename XRaw<T>::load;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const Ld* row = reinterpret_cast<const Ld*>(blk) + (size_t)blockIdx.x * n_out;
-  for (int job = warp; job < n_jobs; job += 8) {
-    const int first = __ldg(jobs + 2 * job), rows = __ldg(jobs + 2 * job + 1);
-    int m = 0;
-#pragma unroll 5
-    for (int r = lane; r < rows; r += 32) m = max(m, x_mag(__ldg(row + first + r)));
-    m = __reduce_max_sync(0xffffffffu, m);
-    // 2^-5 of headroom in the significand: the largest magnitude has to fit
-    // digits whose range is [-64, 63]; a row of zeros or subnormals counts as zero
-    int e;
-    if (std::is_same<T, double>::value) e = m >= 0x7ff00000 ? kXBad : m < 0x100000 ? 0 : ((m + 0x8000) >> 20) - 1022;
-    else e = m >= 0x7f800000 ? kXBad : max(((m + 0x40000) >> 23) - 126, -72);
-    if (lane == 0) E[(size_t)blockIdx.x * n_jobs + job] = e;
+  for (int l = warp; l < n_loads; l += 8) {
+    const int4 p = __ldg(loads + l);  // at most 144 rows
+    int mag[5];
+#pragma unroll
+    for (int i = 0; i < 5; i++) mag[i] = lane + 32 * i < p.y ? x_mag(__ldg(row + p.x + lane + 32 * i)) : 0;
+    for (int job = p.z; job < p.w; job++) {
+      const int2 j = __ldg(jobs + job);
+      int m = 0;
+#pragma unroll
+      for (int i = 0; i < 5; i++) {
+        const int r = lane + 32 * i - j.x;  // three columns: elements 12 i1 + i2, i2 < 3
+        const bool in = j.y == kExactColumns ? r >= 0 && r % 12 < 3 : (unsigned)r < (unsigned)j.y;
+        m = in ? max(m, mag[i]) : m;
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      // 2^-5 of headroom in the significand: the largest magnitude has to fit
+      // digits whose range is [-64, 63]; a row of zeros or subnormals counts as zero
+      int e;
+      if (std::is_same<T, double>::value) e = m >= 0x7ff00000 ? kXBad : m < 0x100000 ? 0 : ((m + 0x8000) >> 20) - 1022;
+      else e = m >= 0x7f800000 ? kXBad : max(((m + 0x40000) >> 23) - 126, -72);
+      if (lane == 0) E[(size_t)blockIdx.x * n_jobs + job] = e;
+    }
   }
 }
 
@@ -915,11 +925,13 @@ static bool exact_set_ok(const ExactDev& S, int form) {
          x_shape(stack, S.nAp, S.nBp).n_stages >= 2;
 }
 
-cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const int* jobs, int n_jobs,
-                                   int* E, cudaStream_t st) {
-  if (n_q <= 0 || n_jobs <= 0) return cudaErrorInvalidValue;
-  if (df) k_exact_exponents<dfr><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, jobs, n_jobs, E);
-  else k_exact_exponents<double><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, jobs, n_jobs, E);
+cudaError_t launch_exact_exponents(const void* blk, bool df, long long n_q, int n_out, const ExactArgs& a, int* E,
+                                   cudaStream_t st) {
+  if (n_q <= 0 || a.n_jobs <= 0) return cudaErrorInvalidValue;
+  if (df)
+    k_exact_exponents<dfr><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, a.loads, a.n_loads, a.jobs, a.n_jobs, E);
+  else
+    k_exact_exponents<double><<<(unsigned)n_q, 256, 0, st>>>(blk, n_out, a.loads, a.n_loads, a.jobs, a.n_jobs, E);
   return cudaGetLastError();
 }
 

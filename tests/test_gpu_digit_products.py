@@ -54,3 +54,19 @@ def test_smooth_fields_in_double_float(bbc, L, eps):
     chans = [0, 16] if L == 8 else list(range(52))
     want = _oracle(L, Sl, Ss, chans) if L == 8 else _run(bbc, L, Sl, Ss, chans, bbc.BBC_FP64)
     assert _err(_run(bbc, L, Sl, Ss, chans, bbc.BBC_DF64), want) <= TOL
+
+
+@pytest.mark.parametrize("w", [0.1, 1e-2, 1e-5])
+@pytest.mark.parametrize("lower", [False, True])
+@pytest.mark.parametrize("chans", [[0, 1, 10, 16, 51], [70, 99, 145, 150]])
+@pytest.mark.parametrize("precision", [0, 3])
+def test_graded_dirac_components(bbc, precision, chans, lower, w):
+    """Lower or upper Dirac components w times the other ones, of the source index alone and of both indices:
+    slices of a block that are far smaller than the block."""
+    L, gen = 4, torch.Generator(device="cuda").manual_seed(8)
+    g = torch.tensor([1.0] * 6 + [w] * 6, device="cuda", dtype=torch.float64)
+    one = torch.ones_like(g)
+    for sink, src in ((one, g), (g, g), (one, g.flip(0)), (g.flip(0), g.flip(0))):
+        Sl, Ss = (_normal(gen, (L ** 3, 12, 12)) * (sink[:, None] * src) for _ in range(2))
+        want = _oracle(L, Sl, Ss, chans, lower)
+        assert _err(_run(bbc, L, Sl, Ss, chans, precision, lower), want) <= TOL
