@@ -73,8 +73,11 @@ typedef enum {
 
 typedef enum {
   BBC_FP64 = 0,      /* blocks, FFTs, contraction and sums in FP64; the block-pair
-                         products as exact products of 7-bit digits of 55-bit fixed-point
-                         values on the tensor cores where the plan allows */
+                         products, where the plan allows, from 7-bit digits of 55-bit
+                         fixed-point values on the tensor cores: an error of about 2^-51
+                         of the product of the two rows' maxima.  A product below 2^-6 of
+                         that bound, or of a row with non-finite values or one below
+                         2^-900, is made in FP64 instead, term by term */
   BBC_MIXED_FP32 = 1, /* blocks, FFTs and block-pair products in FP32 after an exact
                          per-slice power-of-two rescaling of each propagator; the signed
                          sum over Wick diagrams in double-float arithmetic (two FP32
@@ -99,8 +102,9 @@ typedef enum {
   BBC_DF64 = 3,       /* FP64-accurate results from double-float arithmetic
                          (unevaluated sums of two FP32 values, 48-bit significand) on
                          the FP32 pipes: propagators, blocks, FFTs and Wick sums; the
-                         block-pair products as for BBC_FP64; FP64 only to split the
-                         input and to normalise */
+                         block-pair products as for BBC_FP64 (in double-float
+                         where below 2^-7 of the bound, or of a row below 2^-72); FP64
+                         only to split the input and to normalise */
   BBC_MIXED_TF32 = 4  /* trial: as BBC_MIXED_FP32, with the tensor-core operands rounded
                          once to TF32 (10-bit mantissa, round to nearest) instead of
                          split into two TF32 words: a third of the tensor-core work at

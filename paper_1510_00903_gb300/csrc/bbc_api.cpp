@@ -888,7 +888,8 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
     }
     {
       StageScope scope(c, BBC_STAGE_WICK);
-      e = c->exact ? bbc::launch_exact_wick(c->d_P, c->V, c->ex_args, c->prec == BBC_DF64, n_ch * 16, c->d_ct, c->stream)
+      e = c->exact ? bbc::launch_exact_wick(c->d_P, c->lat.L, c->ex_args, c->prec == BBC_DF64, n_ch * 16,
+                                            c->d_blk + (size_t)slot * c->V * p.n_out * 16, p.n_out, c->d_ct, c->stream)
           : c->prec == BBC_DF64
               ? bbc::launch_wick_sums_df(c->d_P, c->lat.L, c->d_cptr, c->d_citem, c->d_ccoef_df, n_ch, c->d_ct,
                                          c->stream)

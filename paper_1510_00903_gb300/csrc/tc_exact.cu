@@ -3,15 +3,19 @@
 // (Sec. 3 Eq. LN.pLLp.FFT: sums over open indices of A(q) B(-q)).
 //
 // Every operand value x of a row with max |x| < 2^e becomes the integer
-// T = round(x 2^(55 - e)), written in eight signed digits of 7 bits, d_i in
-// [-64, 63], T = sum_i d_i 2^(7 (7 - i)).  The digits are small integers in
-// fp16, their products are exact in the FP32 accumulators of tcgen05.mma
-// (kind::f16), and so are the sums: the digit products of one weight ("level"
-// s = i + j) of a complex product of K = 144 terms add up to at most
-// 8 x 288 x 64^2 < 2^24.  Levels 0 .. 7 are kept, an absolute error of
-// about 2^-54 of (row maximum)^2 per product, below the rounding errors of
-// the FP64 sums this replaces; the levels are put together in 64-bit integers
-// and rounded once.  (This is the splitting idea of Ozaki, Ogita, Oishi and
+// T = x 2^(55 - e), cut towards zero (FP64) or to the nearest (double-float) and
+// written in eight signed digits of 7 bits, d_i in [-64, 63], T = sum_i d_i
+// 2^(7 (7 - i)).  The digits are small integers in fp16, their products are exact
+// in the FP32 accumulators of tcgen05.mma (kind::f16), and so are the sums: the
+// digit products of one weight ("level" s = i + j) of a complex product of
+// K = 144 terms add up to at most 8 x 288 x 64^2 < 2^24.  Levels 0 .. 7 are kept,
+// put together in 64-bit integers and rounded once.  The dropped levels leave an
+// error relative to the product of the two rows' maxima, not to the sum of the
+// terms' magnitudes: 7.5 units of 2^-54 of it rms for Gaussian rows, 16 (with a
+// mean of -15) for rows of one sign, 29 at the most in 10^5 emulated products.
+// A product that comes out far below that bound, and any product of a row the
+// fixed point cannot hold, is therefore made again in the blocks' own arithmetic
+// (k_exact_wick).  (This is the splitting idea of Ozaki, Ogita, Oishi and
 // Rump, Numer. Algorithms 59 (2012), with the products on integers.)
 //
 // A digit pair costs 4 real MACs per complex one at 4096 MACs per clock and
@@ -67,7 +71,21 @@ constexpr int kXProd = kXWarps - kXEpi - 1;    // producer warps, after the MMA 
 constexpr int kXMaxStages = 6;
 constexpr int kXCols = 512;                    // all of tensor memory: one CTA per SM
 constexpr int kXFixed = 2048;                  // static shared memory (at most)
-constexpr int kXBad = 0x7fffffff;              // exponent of a row with a NaN or infinite value
+// exponents that are no exponents: a row the digits cannot hold (a NaN or infinite
+// value, or a largest value below 2^kLow) and a row of zeros.  Beside exponents of
+// at most 2^11 a sum of two above kXNone has a bad one, below -kXNone a zero and no
+// bad one.
+constexpr int kXBad = 0x7000, kXZero = -0x3000, kXNone = 0x2000;
+// Per block type: rows and products below 2^kLow and 2^kLowProduct (the digits of
+// an FP64 value are cut by at most 63 bits, double-float scales are FP32 numbers; a
+// product keeps a normal result), and a product below 2^-kFar of the rows'
+// bound is not trusted (k_exact_wick).
+template <typename T>
+struct XLimits;
+template <>
+struct XLimits<double> { static constexpr int kLow = -900, kLowProduct = -900, kFar = 6; };
+template <>
+struct XLimits<dfr> { static constexpr int kLow = -72, kLowProduct = -90, kFar = 7; };
 
 __device__ __forceinline__ uint32_t x_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -382,11 +400,12 @@ __host__ __device__ inline XShape x_shape(int stack, int nAp, int nBp) {
 }  // namespace
 
 // Exponents of one q per CTA: E[q][job] with max |component| over the job's
-// rows below 0.985 2^E (kXBad: a NaN or infinite value among them).  A warp takes a
+// rows below 0.985 2^E, kXBad or kXZero.  A warp takes a
 // piece of rows (a whole block) and, from the same loads, the jobs inside it: HBM bound.
-__device__ __forceinline__ int x_mag(const double2& v) {  // the exponent-carrying words
-  return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+__device__ __forceinline__ int x_mag(double x) {  // the exponent-carrying word, zero only for zeros
+  return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0);
 }
+__device__ __forceinline__ int x_mag(const double2& v) { return max(x_mag(v.x), x_mag(v.y)); }
 __device__ __forceinline__ int x_mag(const float4& v) {  // both words of a double-float count
   return max(__float_as_int(fabsf(v.x) + fabsf(v.y)) & 0x7fffffff, __float_as_int(fabsf(v.z) + fabsf(v.w)) & 0x7fffffff);
 }
@@ -413,10 +432,11 @@ k_exact_exponents(const void* __restrict__ blk, int n_out, const int4* __restric
       }
       m = __reduce_max_sync(0xffffffffu, m);
       // 2^-5 of headroom in the significand: the largest magnitude has to fit
-      // digits whose range is [-64, 63]; a row of zeros or subnormals counts as zero
+      // digits whose range is [-64, 63]
       int e;
-      if (std::is_same<T, double>::value) e = m >= 0x7ff00000 ? kXBad : m < 0x100000 ? 0 : ((m + 0x8000) >> 20) - 1022;
-      else e = m >= 0x7f800000 ? kXBad : max(((m + 0x40000) >> 23) - 126, -72);
+      if (std::is_same<T, double>::value) e = m >= 0x7ff00000 ? kXBad : ((m + 0x8000) >> 20) - 1022;
+      else e = m >= 0x7f800000 ? kXBad : ((m + 0x40000) >> 23) - 126;
+      e = m == 0 ? kXZero : e < XLimits<T>::kLow ? kXBad : e;
       if (lane == 0) E[(size_t)blockIdx.x * n_jobs + job] = e;
     }
   }
@@ -480,6 +500,15 @@ k_exact_small(const void* __restrict__ blk, int L, int n_out, const DevTask* __r
 // took 93 us (double-float, 16^3, 52 channels).
 // FP64; double-float with the coefficients split on the host, renormalised
 // every 16 terms.
+//
+// Before the sums, products marked NaN are made again, a warp each, from the rows
+// in the blocks' own arithmetic: rows the digits do not hold, and products far
+// below the product of their rows' largest magnitudes.  The digits' error is about
+// 2^-51 of that bound (dropped levels and cut values): 2^-45 of a product at 2^-6 of
+// it, what bounds an FP64 sum of 288 terms; 2^-44, the operators' own error, at 2^-7
+// in double-float.  Where the large values of two rows meet (any field whose
+// flavours are graded alike) under 0.1% of the products are made again; rows graded
+// against each other would lose theirs without it.
 constexpr int kWickThreads = 256;
 struct WickAcc64 {
   double x = 0, y = 0;
@@ -505,14 +534,79 @@ struct WickAccDf {
     return make_float4(re.s, re.e, im.s, im.e);
   }
 };
-template <typename T, typename C, typename Acc>
-__global__ void __launch_bounds__(kWickThreads)
+// Product of the rows a and c of a task by one warp (the result in every lane),
+// kTerms per lane on their way together (as the registers of five CTAs per SM allow).
+struct WarpSum64 {
+  static constexpr int kTerms = 3;
+  cpx<double> acc = cpx<double>(0, 0);
+  __device__ __forceinline__ void mac(double2 x, double2 y) { cmac(acc, cpx<double>(x.x, x.y), cpx<double>(y.x, y.y)); }
+  __device__ __forceinline__ void join(int d) {
+    acc.re += __shfl_xor_sync(0xffffffffu, acc.re, d);
+    acc.im += __shfl_xor_sync(0xffffffffu, acc.im, d);
+  }
+  __device__ __forceinline__ double2 value() { return make_double2(acc.re, acc.im); }
+};
+struct WarpSumDf {
+  static constexpr int kTerms = 2;
+  df64acc re{0.f, 0.f}, im{0.f, 0.f};
+  __device__ __forceinline__ void mac(float4 x, float4 y) {
+    df_mac(re, x.x, x.y, y.x, y.y);
+    df_mac(re, -x.z, -x.w, y.z, y.w);
+    df_mac(im, x.x, x.y, y.z, y.w);
+    df_mac(im, x.z, x.w, y.x, y.y);
+  }
+  __device__ __forceinline__ void join(df64acc& v, int d) {
+    const float s = __shfl_xor_sync(0xffffffffu, v.s, d), e = __shfl_xor_sync(0xffffffffu, v.e, d);
+    float t;
+    two_sum(v.s, s, v.s, t);
+    v.e = __fadd_rn(__fadd_rn(v.e, e), t);
+  }
+  __device__ __forceinline__ void join(int d) {
+    join(re, d);
+    join(im, d);
+  }
+  __device__ __forceinline__ float4 value() {
+    df_renorm(re);
+    df_renorm(im);
+    return make_float4(re.s, re.e, im.s, im.e);
+  }
+};
+template <typename Sum, typename Ld>
+__device__ __forceinline__ Ld x_again(const Ld* rq, const Ld* rn, const DevTask* task, int i) {
+  static_assert(sizeof(DevTask) == 21 * sizeof(int), "fields by position");
+  const int lane = threadIdx.x & 31;
+  const int f = lane < 21 ? __ldg(reinterpret_cast<const int*>(task) + lane) : 0;  // the task in one load
+  auto field = [&](int at) { return __shfl_sync(0xffffffffu, f, at); };
+  const int nB = field(16) >> 8, n2 = field(18), K = field(17) * n2, sA = field(19), sB = field(20);
+  const Ld *a = rq + field(i / nB), *c = rn + field(8 + i % nB);
+  Sum sum;
+  constexpr int n = Sum::kTerms;
+  for (int k0 = lane; k0 < K; k0 += 32 * n) {
+    Ld x[n], y[n];
+#pragma unroll
+    for (int j = 0; j < n; j++) {
+      const int k = min(k0 + 32 * j, K - 1), i1 = k / n2, i2 = k - i1 * n2;
+      x[j] = __ldg(a + i1 * (sA & 0xffff) + i2 * (sA >> 16));
+      y[j] = __ldg(c + i1 * (sB & 0xffff) + i2 * (sB >> 16));
+    }
+#pragma unroll
+    for (int j = 0; j < n; j++)
+      if (k0 + 32 * j < K) sum.mac(x[j], y[j]);
+  }
+#pragma unroll
+  for (int d = 16; d; d >>= 1) sum.join(d);
+  return sum.value();
+}
+template <typename T, typename C, typename Acc, typename Sum>
+__global__ void __launch_bounds__(kWickThreads, 5)
 k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* __restrict__ coefs, int n_outputs,
+             const void* __restrict__ blk, int L, int n_out, const DevTask* __restrict__ tasks,
              void* __restrict__ ct) {
   using Ld = typename XRaw<T>::load;
   extern __shared__ __align__(128) unsigned char smem[];
   Ld* s_p = reinterpret_cast<Ld*>(smem);                                // [n_items]
   C* s_c = reinterpret_cast<C*>(smem + (size_t)n_items * sizeof(Ld));  // [n_coefs]
+  uint32_t* s_again = reinterpret_cast<uint32_t*>(s_c + W.n_coefs);     // a bit per item
   const int q = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   {
     const Ld* src = reinterpret_cast<const Ld*>(P) + (size_t)q * n_items;
@@ -520,7 +614,33 @@ k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* 
     for (int i = threadIdx.x; i < W.n_coefs; i += kWickThreads) s_c[i] = __ldg(coefs + i);
     cp_async_wait_all();
   }
-  __syncthreads();
+  bool any = false;
+  for (int i0 = 32 * warp; i0 < n_items; i0 += kWickThreads) {  // (each thread's own copies)
+    const int i = i0 + lane;
+    const uint32_t bits = __ballot_sync(0xffffffffu, i < n_items && s_p[i].x != s_p[i].x);
+    if (lane == 0) s_again[i0 >> 5] = bits;
+    any |= bits != 0;
+  }
+  if (__syncthreads_or(any)) {
+    const Ld* F = reinterpret_cast<const Ld*>(blk);
+    const Ld *rq = F + (size_t)q * n_out, *rn = F + (size_t)x_neg_site(q, L) * n_out;
+    // a warp takes every eighth marked product (they come in runs and patterns)
+    const int words = (n_items + 31) / 32;
+    int n = 0;
+    for (int w0 = 0; w0 < words; w0 += 32) {
+      const uint32_t word = w0 + lane < words ? s_again[w0 + lane] : 0;
+      for (uint32_t live = __ballot_sync(0xffffffffu, word != 0); live; live &= live - 1) {
+        const int l = __ffs((int)live) - 1;
+        for (uint32_t bits = __shfl_sync(0xffffffffu, word, l); bits; bits &= bits - 1)
+          if (n++ % (kWickThreads / 32) == warp) {
+            const int item = 32 * (w0 + l) + __ffs((int)bits) - 1;
+            const Ld v = x_again<Sum>(rq, rn, tasks + (item >> 4), item & 15);
+            if (lane == 0) s_p[item] = v;
+          }
+      }
+    }
+    __syncthreads();
+  }
   for (int c = warp; c < W.n_chunks; c += kWickThreads / 32) {
     const Ld* p = s_p;
     const int2 ch = __ldg(W.chunks + c);  // offset, terms of the longest output
@@ -643,7 +763,7 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       if (row < (sideB ? S.nB : S.nA)) {
         const Ld* p = F + (size_t)q * n_out + __ldg((sideB ? S.rowB : S.rowA) + row);
         e = __ldg(E + (size_t)q * n_jobs + __ldg((sideB ? S.expB : S.expA) + row));
-        e = e == kXBad ? 0 : e;  // any digits: the epilogue writes NaN
+        e = abs(e) > kXNone ? 0 : e;  // any digits, or zeros
         if (STACK == 2) {
           // chunk c is the 4 x 4 tile (u, v) = (4 tu .., 4 tv ..) of the open
           // indices, k-group kg its u = 4 tu + 2 kg + (0, 1): values j = 4 du + dv
@@ -804,9 +924,8 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       const int buf = n_buf == 2 ? i & 1 : 0, m = n_buf == 2 ? i >> 1 : i;
       short* s_ex = xs.ex[i & 1];
       short* s_ey = xs.ey[i & 1];
-      // |exponent| < 2^11 (kXBad: 2^15 - 1)
-      if (tid < S.nA) s_ex[tid] = (short)min(ex_next, 0x7fff);
-      if (tid < S.nB) s_ey[tid] = (short)min(ey_next, 0x7fff);
+      if (tid < S.nA) s_ex[tid] = (short)ex_next;
+      if (tid < S.nB) s_ey[tid] = (short)ey_next;
       Ld* pq = reinterpret_cast<Ld*>(P) + (size_t)q * n_items;
       Ld* pn = reinterpret_cast<Ld*>(P) + (size_t)nq * n_items;
       const bool self = STACK == 2 && nq == q;  // q = -q has its products from the items at q
@@ -857,9 +976,12 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
           re += p[2 * NB * S.nAp];
           im += p[3 * NB * S.nAp];
         }
-        // the sum is (sum of T_A T_B) 2^-56, T = x 2^(55 - e)
-        const int ex = s_ex[row], ey = s_ey[col];
-        const Ld v = x_value(Ld(), re, im, ex == 0x7fff || ey == 0x7fff ? kXBad : ex + ey - 54);
+        // the sum is (sum of T_A T_B) 2^-56, T = x 2^(55 - e): 2^54 stands for the
+        // product of the rows' bounds.  NaN marks what k_exact_wick makes again.
+        const int e = s_ex[row] + s_ey[col], hr = (int)(re >> 32), hi = (int)(im >> 32);
+        const bool far = max(hr ^ (hr >> 31), hi ^ (hi >> 31)) < (1 << (22 - XLimits<T>::kFar));
+        const bool again = e > kXNone || (e >= -kXNone && (far || e < XLimits<T>::kLowProduct));
+        const Ld v = x_value(Ld(), re, im, again ? kXBad : e - 54);
         const int item_q = (int)(short)en.y, item_n = en.y >> 16;
         if (item_q >= 0) pq[item_q] = v;
         if (item_n >= 0 && !self) pn[item_n] = v;
@@ -981,25 +1103,28 @@ cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, co
             : launch_exact_t<double>(blk, L, n_out, a, E, qlist, n_pairs, P, err, spin_limit, n_sm[dev], st);
 }
 
-static size_t wick_smem(int n_items, int n_coefs) { return 16 * (size_t)n_items + (((size_t)n_coefs * 8 + 15) & ~(size_t)15); }
+static size_t wick_smem(int n_items, int n_coefs) {
+  return 16 * (size_t)n_items + 8 * (size_t)n_coefs + 4 * (((size_t)n_items + 31) / 32);
+}
 bool exact_wick_fits(int n_items, int n_coefs) { return wick_smem(n_items, n_coefs) <= kMaxSmemPerBlock; }
 
-template <typename T, typename C, typename Acc>
-static cudaError_t launch_wick_t(const void* P, int V, const ExactArgs& a, const C* coefs, int n_outputs, void* ct,
-                                 cudaStream_t st) {
+template <typename T, typename C, typename Acc, typename Sum>
+static cudaError_t launch_wick_t(const void* P, int L, const ExactArgs& a, const C* coefs, int n_outputs,
+                                 const void* blk, int n_out, void* ct, cudaStream_t st) {
   const size_t sm = wick_smem(a.n_items, a.wick.n_coefs);
   if (sm > kMaxSmemPerBlock) return cudaErrorInvalidValue;
   static int granted[64] = {0};
-  const cudaError_t e = ensure_smem(k_exact_wick<T, C, Acc>, sm, granted);
+  const cudaError_t e = ensure_smem(k_exact_wick<T, C, Acc, Sum>, sm, granted);
   if (e != cudaSuccess) return e;
-  k_exact_wick<T, C, Acc><<<(unsigned)V, kWickThreads, sm, st>>>(P, a.n_items, a.wick, coefs, n_outputs, ct);
+  k_exact_wick<T, C, Acc, Sum><<<(unsigned)(L * L * L), kWickThreads, sm, st>>>(P, a.n_items, a.wick, coefs, n_outputs, blk,
+                                                                           L, n_out, a.tasks, ct);
   return cudaGetLastError();
 }
 
-cudaError_t launch_exact_wick(const void* P, int V, const ExactArgs& a, bool df, int n_outputs, void* ct,
-                              cudaStream_t st) {
-  return df ? launch_wick_t<dfr, float2, WickAccDf>(P, V, a, a.wick.coefs_df, n_outputs, ct, st)
-            : launch_wick_t<double, double, WickAcc64>(P, V, a, a.wick.coefs, n_outputs, ct, st);
+cudaError_t launch_exact_wick(const void* P, int L, const ExactArgs& a, bool df, int n_outputs, const void* blk,
+                              int n_out, void* ct, cudaStream_t st) {
+  return df ? launch_wick_t<dfr, float2, WickAccDf, WarpSumDf>(P, L, a, a.wick.coefs_df, n_outputs, blk, n_out, ct, st)
+            : launch_wick_t<double, double, WickAcc64, WarpSum64>(P, L, a, a.wick.coefs, n_outputs, blk, n_out, ct, st);
 }
 
 }  // namespace bbc

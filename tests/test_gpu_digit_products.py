@@ -70,3 +70,48 @@ def test_graded_dirac_components(bbc, precision, chans, lower, w):
         Sl, Ss = (_normal(gen, (L ** 3, 12, 12)) * (sink[:, None] * src) for _ in range(2))
         want = _oracle(L, Sl, Ss, chans, lower)
         assert _err(_run(bbc, L, Sl, Ss, chans, precision, lower), want) <= TOL
+
+
+# (double-float has FP32's range: a block of three quarks of 1e-20 underflows in its arithmetic)
+@pytest.mark.parametrize("precision,w", [(0, 1e-2), (0, 1e-4), (0, 1e-20), (3, 1e-2), (3, 1e-4)])
+@pytest.mark.parametrize("lower", [False, True])
+def test_flavours_graded_against_each_other(bbc, precision, lower, w):
+    """Light quarks from upper, strange quarks from lower Dirac components: the large values of one row meet the
+    small ones of the other, and products lie far below what their rows' maxima suggest."""
+    L, chans, gen = 4, [0, 1, 10, 16, 51, 70, 145, 150], torch.Generator(device="cuda").manual_seed(9)
+    g = torch.tensor([1.0] * 6 + [w] * 6, device="cuda", dtype=torch.float64)
+    for gl, gs in ((g, g.flip(0)), (g.flip(0), g)):
+        Sl, Ss = _normal(gen, (L ** 3, 12, 12)) * gl, _normal(gen, (L ** 3, 12, 12)) * gs
+        assert _err(_run(bbc, L, Sl, Ss, chans, precision, lower), _oracle(L, Sl, Ss, chans, lower)) <= TOL
+
+
+@pytest.mark.parametrize("chans", [list(range(52)), list(range(64, 154, 7))])
+@pytest.mark.parametrize("precision", [0, 3])
+def test_products_that_vanish_term_by_term(bbc, precision, chans):
+    """Propagators diagonal in colour (unit gauge links): most terms of every product are exact zeros."""
+    L, gen = 4, torch.Generator(device="cuda").manual_seed(10)
+    Sl, Ss = (torch.einsum("vab,cd->vacbd", _normal(gen, (L ** 3, 4, 4)),
+                           torch.eye(3, dtype=torch.complex128, device="cuda")).reshape(L ** 3, 12, 12).contiguous()
+              for _ in range(2))
+    want = _oracle(L, Sl, Ss, chans)
+    scale = want.abs().amax()
+    got = _run(bbc, L, Sl, Ss, chans, precision)
+    live = want.abs().flatten(1).amax(1) > 1e-9 * scale
+    assert live.any() and _err(got[live], want[live]) <= TOL
+    assert ((got - want)[~live].abs() <= TOL * scale).all()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("precision", [0, 3])
+def test_non_finite_values_reach_what_reads_them(bbc, precision, value):
+    """A non-finite light entry spoils every channel, a strange one those with strange quarks and no other."""
+    L, chans, gen = 4, [0, 1, 16, 51], torch.Generator(device="cuda").manual_seed(11)
+    Sl, Ss = (_normal(gen, (L ** 3, 12, 12)) for _ in range(2))
+    bad = [S.clone() for S in (Sl, Ss)]
+    for S in bad:
+        S[5, 3, 4] = value
+    got = _run(bbc, L, bad[0], Ss, chans, precision)
+    assert (~torch.isfinite(torch.view_as_real(got))).flatten(1).any(1).all()
+    got = _run(bbc, L, Sl, bad[1], chans, precision)
+    assert (~torch.isfinite(torch.view_as_real(got[1:]))).flatten(1).any(1).all()
+    assert _err(got[:1], _oracle(L, Sl, Ss, chans[:1])) <= TOL
