@@ -293,9 +293,12 @@ bbc_status bbc_set_checks(bbc_ctx* ctx, int flags);
  * z plane) and (row tile, z lines) units from a device work queue; a z-lines
  * unit waits for the planes of its row tile, at most about a second, and a
  * wait that gives up sets a sticky device word and stops the launch.  The
- * tensor-core contraction of the mixed precisions (one persistent CTA per SM,
+ * tensor-core contraction of the mixed precisions and the digit-sliced products
+ * of BBC_FP64 and BBC_DF64 (one persistent CTA per SM,
  * tcgen05 products committed to mbarriers) bounds its mbarrier waits the
- * same way and sets another bit of the word.  bbc_device_status synchronises
+ * same way and sets another bit of the word; the BBC_FP64 and BBC_DF64
+ * correlators of that contraction, and of later ones until the word is read, are
+ * then NaN.  bbc_device_status synchronises
  * the context stream and returns BBC_ETIMEOUT if either happened since the
  * last call (the word is cleared; after an FFT timeout every slot is marked
  * unbuilt, its blocks not being valid; after a contraction timeout the
@@ -313,6 +316,14 @@ bbc_status bbc_device_status(bbc_ctx* ctx);
  * workspace or without the queue-driven FFT (FP64, double-float, L = 48, or
  * a plan too large for the fused kernels).  Not inside a stream capture. */
 bbc_status bbc_check_bounded_wait(bbc_ctx* ctx, long long spin_limit);
+
+/* Self-test of the waits of the digit-sliced products (BBC_FP64, BBC_DF64): the
+ * products of slot 0's blocks with at most spin_limit (1 .. 2^22) polls per wait.
+ * Synchronous.  Returns BBC_ETIMEOUT when a wait gave up (the expected outcome of
+ * a limit of 1; the context stays usable), BBC_OK when none did, EINVAL for
+ * spin_limit out of range, ESTATE without a workspace, without built blocks or in a
+ * context whose products run elsewhere.  Not inside a stream capture. */
+bbc_status bbc_check_products_wait(bbc_ctx* ctx, long long spin_limit);
 
 /* Launch configuration of the two kernels whose shape is tunable:
  *  build_sites, build_threads: sites per CTA and threads of the block build,

@@ -115,6 +115,7 @@ def _load():
         "bbc_set_checks": ([P, I], I),
         "bbc_device_status": ([P], I),
         "bbc_check_bounded_wait": ([P, LL], I),
+        "bbc_check_products_wait": ([P, LL], I),
         "bbc_batch_run": ([ctypes.POINTER(bbc_batch_item), I, P, ctypes.POINTER(I)], I),
         "bbc_get_tuning": ([P, ctypes.POINTER(bbc_tuning)], I),
         "bbc_set_tuning": ([P, ctypes.POINTER(bbc_tuning)], I),
@@ -312,6 +313,11 @@ def bbc_check_bounded_wait(ctx, spin_limit: int) -> int:
     return int(_lib.bbc_check_bounded_wait(ctx, int(spin_limit)))
 
 
+def bbc_check_products_wait(ctx, spin_limit: int) -> int:
+    """Self-test of the waits of the digit-sliced products on slot 0; returns the status (BBC_ETIMEOUT expected)."""
+    return int(_lib.bbc_check_products_wait(ctx, int(spin_limit)))
+
+
 def bbc_get_tuning(ctx) -> dict:
     t = bbc_tuning()
     _check(ctx, _lib.bbc_get_tuning(ctx, ctypes.byref(t)))
@@ -408,6 +414,8 @@ class Correlators:
         bbc_contract(self.ctx, slot, out.data_ptr(), normalised)
 
     def run(self, S_light, S_strange, times, out=None, normalised: bool = True):
+        """Correlators [len(times), n_ch, L^3, 16] of the slices.  Asynchronous: a device wait that gave up is
+        seen by status() (and as NaN in FP64 and double-float)."""
         torch = self.torch
         times = list(times)
         n_ch = len(self.channels)

@@ -331,11 +331,11 @@ cudaError_t launch_build(bbc_ctx* c, int n_slots, int sites, int threads) {
 }
 
 // The digit-sliced products of one slot into P.
-cudaError_t launch_exact(bbc_ctx* c, int slot) {
+cudaError_t launch_exact(bbc_ctx* c, int slot, long long spin_limit = bbc::kFftSpinLimit) {
   return bbc::launch_contract_exact(c->d_blk + (size_t)slot * c->V * c->plan.n_out * 16, c->lat.L, c->plan.n_out,
                                     c->prec == BBC_DF64, c->ex_args,
                                     c->d_exE + (size_t)slot * c->V * c->ex_args.n_jobs, c->d_qlist,
-                                    (int)c->qlist.size(), c->d_P, c->d_qerr, bbc::kFftSpinLimit, c->stream);
+                                    (int)c->qlist.size(), c->d_P, c->d_qerr, spin_limit, c->stream);
 }
 
 // The tensor-core contraction of one slot: G(q) of every pair {q, -q} on
@@ -889,7 +889,8 @@ bbc_status bbc_contract(bbc_ctx* c, int slot, void* out_dev, int normalised) {
     {
       StageScope scope(c, BBC_STAGE_WICK);
       e = c->exact ? bbc::launch_exact_wick(c->d_P, c->lat.L, c->ex_args, c->prec == BBC_DF64, n_ch * 16,
-                                            c->d_blk + (size_t)slot * c->V * p.n_out * 16, p.n_out, c->d_ct, c->stream)
+                                            c->d_blk + (size_t)slot * c->V * p.n_out * 16, p.n_out, c->d_qerr, c->d_ct,
+                                            c->stream)
           : c->prec == BBC_DF64
               ? bbc::launch_wick_sums_df(c->d_P, c->lat.L, c->d_cptr, c->d_citem, c->d_ccoef_df, n_ch, c->d_ct,
                                          c->stream)
@@ -959,6 +960,17 @@ bbc_status bbc_check_bounded_wait(bbc_ctx* c, long long spin_limit) {
                                                 bbc::FftQueue{c->d_fftq, c->d_qerr}, c->lat.L + 1, spin_limit,
                                                 c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "bounded-wait self-test");
+  return wait_status(c);
+}
+
+bbc_status bbc_check_products_wait(bbc_ctx* c, long long spin_limit) {
+  if (!c) return BBC_EINVAL;
+  if (spin_limit < 1 || spin_limit > bbc::kFftSpinLimit) return fail(c, BBC_EINVAL, "spin_limit outside [1, 2^22]");
+  if (!c->ws) return fail(c, BBC_ESTATE, "no workspace attached");
+  if (!c->exact) return fail(c, BBC_ESTATE, "this context has no digit-sliced products");
+  if (!c->slot_built[0]) return fail(c, BBC_ESTATE, "slot 0 has no blocks");
+  cudaError_t e = launch_exact(c, 0, spin_limit);
+  if (e != cudaSuccess) return cuda_fail(c, e, "products' wait self-test");
   return wait_status(c);
 }
 

@@ -212,7 +212,8 @@ cudaError_t launch_fft_inverse_df(void* ct, void* out, int L, int n_ch, const do
 // the operands' exponents E[n_q][n_jobs] (one per operand row and q), the
 // products (small tasks one product per thread, then the trace sets per pair
 // {q, -q} of qlist[n_pairs] and the slice sets per q; NaN: to be made again) and the
-// signed sums over Wick diagrams into ct[V][n_outputs] (which makes them again from blk).  The mbarrier waits give up after
+// signed sums over Wick diagrams into ct[V][n_outputs] (which makes them again from blk;
+// NaN while bit 1 of *err is set).  The mbarrier waits give up after
 // spin_limit polls and set bit 1 of *err.
 constexpr int kExactMaxBlocks = 48;   // blocks of a trace set (its sums and three stages fill shared memory)
 constexpr int kExactMaxSliceA = 128;  // rows of one instruction
@@ -253,7 +254,7 @@ cudaError_t launch_contract_exact(const void* blk, int L, int n_out, bool df, co
                                   cudaStream_t st);
 bool exact_wick_fits(int n_items, int n_coefs);
 cudaError_t launch_exact_wick(const void* P, int L, const ExactArgs& a, bool df, int n_outputs, const void* blk,
-                              int n_out, void* ct, cudaStream_t st);
+                              int n_out, const int* err, void* ct, cudaStream_t st);
 // ... then the signed FP64 sums over Wick diagrams into ct[n_ch*16][V] (complex128).
 cudaError_t launch_wick_sums(const void* P, int L, const int* cptr, const int* citem, const double* ccoef, int n_ch,
                              void* ct, bool fp64, cudaStream_t st);

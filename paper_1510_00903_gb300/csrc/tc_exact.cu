@@ -50,8 +50,9 @@
 // lie in two runs of n_out values), split them and store the digits in the canonical K-major
 // layout without swizzle, 16 open indices per stage of an mbarrier ring.
 // Every wait is bounded: past its limit, or when another warp gave up, the
-// warps leave their loops, the MMAs in flight are waited for (bounded), the
-// tensor memory is freed and bit 1 of the error word is set.
+// warps leave their loops, the MMAs in flight are waited for (a limit of its own), the
+// tensor memory is freed and bit 1 of the error word is set; k_exact_wick then
+// writes NaN, until the host has read the word.
 #include <algorithm>
 #include <type_traits>
 
@@ -69,6 +70,7 @@ constexpr int kXWarps = 20;
 constexpr int kXEpi = 8;                       // epilogue warps (tensor-memory lanes 32 (w mod 4) .., column chunks w / 4)
 constexpr int kXProd = kXWarps - kXEpi - 1;    // producer warps, after the MMA warp
 constexpr int kXMaxStages = 6;
+constexpr long long kXDrainLimit = 1ll << 22;  // polls for the MMAs in flight (about a second)
 constexpr int kXCols = 512;                    // all of tensor memory: one CTA per SM
 constexpr int kXFixed = 2048;                  // static shared memory (at most)
 // exponents that are no exponents: a row the digits cannot hold (a NaN or infinite
@@ -601,7 +603,7 @@ template <typename T, typename C, typename Acc, typename Sum>
 __global__ void __launch_bounds__(kWickThreads, 5)
 k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* __restrict__ coefs, int n_outputs,
              const void* __restrict__ blk, int L, int n_out, const DevTask* __restrict__ tasks,
-             void* __restrict__ ct) {
+             const int* __restrict__ err, void* __restrict__ ct) {
   using Ld = typename XRaw<T>::load;
   extern __shared__ __align__(128) unsigned char smem[];
   Ld* s_p = reinterpret_cast<Ld*>(smem);                                // [n_items]
@@ -614,6 +616,7 @@ k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* 
     for (int i = threadIdx.x; i < W.n_coefs; i += kWickThreads) s_c[i] = __ldg(coefs + i);
     cp_async_wait_all();
   }
+  const bool lost = __ldg(err) & 2;  // a wait of the products gave up: they are not valid
   bool any = false;
   for (int i0 = 32 * warp; i0 < n_items; i0 += kWickThreads) {  // (each thread's own copies)
     const int i = i0 + lane;
@@ -659,7 +662,7 @@ k_exact_wick(const void* __restrict__ P, int n_items, const WickDev W, const C* 
         if (j0 + j < out.y) acc.add(s_c[e[j] >> 16], v[j]);
       if ((j0 & 12) == 12) acc.renorm();  // every 16 terms
     }
-    if (out.x >= 0) reinterpret_cast<Ld*>(ct)[(size_t)q * n_outputs + out.x] = acc.value();
+    if (out.x >= 0) reinterpret_cast<Ld*>(ct)[(size_t)q * n_outputs + out.x] = lost ? x_value(Ld(), 0, 0, kXBad) : acc.value();
   }
 }
 
@@ -889,10 +892,13 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
       }
       if (!ok) break;
     }
-    // every MMA issued has finished before the tensor memory is freed
+    // every MMA issued has finished before the tensor memory is freed, also when a
+    // wait above gave up early; this wait has its own, long limit
     if (leader) {
       x_commit(bar_drain);
-      for (long long polls = 0; !x_test(bar_drain, 0) && polls < spin_limit; polls++) __nanosleep(20);
+      long long polls = 0;
+      for (; !x_test(bar_drain, 0) && polls < kXDrainLimit; polls++) __nanosleep(20);
+      if (polls == kXDrainLimit) *abort_flag = 1;
     }
     __syncwarp();
   } else {
@@ -1110,21 +1116,21 @@ bool exact_wick_fits(int n_items, int n_coefs) { return wick_smem(n_items, n_coe
 
 template <typename T, typename C, typename Acc, typename Sum>
 static cudaError_t launch_wick_t(const void* P, int L, const ExactArgs& a, const C* coefs, int n_outputs,
-                                 const void* blk, int n_out, void* ct, cudaStream_t st) {
+                                 const void* blk, int n_out, const int* err, void* ct, cudaStream_t st) {
   const size_t sm = wick_smem(a.n_items, a.wick.n_coefs);
   if (sm > kMaxSmemPerBlock) return cudaErrorInvalidValue;
   static int granted[64] = {0};
   const cudaError_t e = ensure_smem(k_exact_wick<T, C, Acc, Sum>, sm, granted);
   if (e != cudaSuccess) return e;
   k_exact_wick<T, C, Acc, Sum><<<(unsigned)(L * L * L), kWickThreads, sm, st>>>(P, a.n_items, a.wick, coefs, n_outputs, blk,
-                                                                           L, n_out, a.tasks, ct);
+                                                                           L, n_out, a.tasks, err, ct);
   return cudaGetLastError();
 }
 
 cudaError_t launch_exact_wick(const void* P, int L, const ExactArgs& a, bool df, int n_outputs, const void* blk,
-                              int n_out, void* ct, cudaStream_t st) {
-  return df ? launch_wick_t<dfr, float2, WickAccDf, WarpSumDf>(P, L, a, a.wick.coefs_df, n_outputs, blk, n_out, ct, st)
-            : launch_wick_t<double, double, WickAcc64, WarpSum64>(P, L, a, a.wick.coefs, n_outputs, blk, n_out, ct, st);
+                              int n_out, const int* err, void* ct, cudaStream_t st) {
+  return df ? launch_wick_t<dfr, float2, WickAccDf, WarpSumDf>(P, L, a, a.wick.coefs_df, n_outputs, blk, n_out, err, ct, st)
+            : launch_wick_t<double, double, WickAcc64, WarpSum64>(P, L, a, a.wick.coefs, n_outputs, blk, n_out, err, ct, st);
 }
 
 }  // namespace bbc

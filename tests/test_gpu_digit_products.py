@@ -115,3 +115,31 @@ def test_non_finite_values_reach_what_reads_them(bbc, precision, value):
     got = _run(bbc, L, Sl, bad[1], chans, precision)
     assert (~torch.isfinite(torch.view_as_real(got[1:]))).flatten(1).any(1).all()
     assert _err(got[:1], _oracle(L, Sl, Ss, chans[:1])) <= TOL
+
+
+@pytest.mark.parametrize("chans", [[0], list(range(52)), [64, 70, 99, 145]])
+@pytest.mark.parametrize("precision", [0, 3])
+def test_products_waits_run_out_and_the_context_recovers(bbc, precision, chans):
+    """With one poll per wait the first waits give up: the kernel records it, frees its tensor memory and returns,
+    and the context stays usable."""
+    L, gen = 4, torch.Generator(device="cuda").manual_seed(12)
+    Sl, Ss = (_normal(gen, (1, L ** 3, 12, 12)) for _ in range(2))
+    cor = bbc.Correlators(L, 4, 0, 0.3, 0.4, channels=chans, precision=precision)
+    assert bbc.bbc_check_products_wait(cor.ctx, 1) == bbc.BBC_ESTATE  # nothing built
+    before = cor.run(Sl, Ss, [0]).clone()
+    cor.status()
+    for _ in range(3):
+        assert bbc.bbc_check_products_wait(cor.ctx, 1) == bbc.BBC_ETIMEOUT
+        assert "bounded wait" in bbc.lib().bbc_last_error(cor.ctx).decode()
+    cor.status()  # the record was read and cleared
+    assert bbc.bbc_check_products_wait(cor.ctx, 1 << 22) == bbc.BBC_OK
+    assert torch.equal(cor.run(Sl, Ss, [0]), before)
+    cor.status()
+    cor.close()
+
+
+def test_products_wait_self_test_needs_the_digit_products(bbc):
+    cor = bbc.Correlators(4, 4, 0, 0.3, 0.4, channels=[0], precision=bbc.BBC_MIXED_FP32)
+    assert bbc.bbc_check_products_wait(cor.ctx, 1) == bbc.BBC_ESTATE
+    assert bbc.bbc_check_products_wait(cor.ctx, 0) == bbc.BBC_EINVAL
+    cor.close()
