@@ -195,6 +195,12 @@ bbc_status bbc_plan_stats(const bbc_ctx* ctx, int channel_pos, int term3, int te
 bbc_status bbc_plan_sizes(const bbc_ctx* ctx, int* n_blocks, int* n_block_outputs,
                           int* n_pair_items, long long* pair_macs_per_site);
 
+/* 1 if the block-pair products of this context (BBC_FP64, BBC_DF64) are the
+ * digit-sliced ones on the tensor cores, 0 if they run on the CUDA cores: plans
+ * the digit kernel does not hold, and lists of few channels on larger lattices,
+ * which the CUDA cores serve faster. */
+int bbc_digit_products(const bbc_ctx* ctx);
+
 /* The whole contraction plan as host tables (no device work), so that a host
  * program can evaluate the block algorithm of Sec. 3 step by step (the tests
  * do, on tiny lattices, against the oracle).  Call once with every array

@@ -106,6 +106,7 @@ def _load():
         "bbc_contract": ([P, I, P, I], I),
         "bbc_plan_stats": ([P, I, I, I, ctypes.POINTER(I), ctypes.POINTER(I), I], I),
         "bbc_plan_sizes": ([P, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(LL)], I),
+        "bbc_digit_products": ([P], I),
         "bbc_plan_export": ([P, P, P, P, P, P, P, P], I),
         "bbc_enable_stage_timing": ([P, I], I),
         "bbc_stage_timing": ([P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(LL)], I),
@@ -200,6 +201,11 @@ def bbc_plan_sizes(ctx):
     a, b, c, d = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_longlong()
     _check(ctx, _lib.bbc_plan_sizes(ctx, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c), ctypes.byref(d)))
     return {"blocks": a.value, "block_outputs": b.value, "pair_items": c.value, "pair_macs_per_site": d.value}
+
+
+def bbc_digit_products(ctx) -> bool:
+    """Whether the block-pair products run as digit-sliced products on the tensor cores."""
+    return bool(_lib.bbc_digit_products(ctx))
 
 
 def bbc_plan_export(ctx) -> dict:

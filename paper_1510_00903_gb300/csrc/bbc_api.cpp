@@ -462,7 +462,8 @@ bbc_status bbc_create_components(bbc_ctx** ctx, const bbc_lattice* lat, bbc_prec
       delete c;
       return fail(nullptr, BBC_ENOMEM, "host allocation failed while scheduling");
     }
-    c->exact = c->ex.all && bbc::exact_wick_fits(16 * (int)c->plan.tasks.size(), (int)c->ex.wick_coefs.size());
+    c->exact = c->ex.all && bbc::exact_wick_fits(16 * (int)c->plan.tasks.size(), (int)c->ex.wick_coefs.size()) &&
+               bbc::exact_pays(c->plan, c->ex, c->lat.L, prec == BBC_DF64);
   }
   // Block build of the FP64-accurate precisions: where shared memory holds at
   // most two one-site CTAs per SM (two octet diquarks and 4548 tensor entries: 89 KB),
@@ -1210,6 +1211,8 @@ bbc_status bbc_plan_sizes(const bbc_ctx* c, int* n_blocks, int* n_block_outputs,
   if (pair_macs_per_site) *pair_macs_per_site = c->plan.pair_macs;
   return BBC_OK;
 }
+
+int bbc_digit_products(const bbc_ctx* c) { return c && c->exact ? 1 : 0; }
 
 bbc_status bbc_plan_export(const bbc_ctx* c, int* sizes, int* row_ptr, int* terms, int* tasks, int* out_ptr,
                            int* items, double* coefs) {

@@ -13,8 +13,9 @@
 // Every product the tasks need gets its place in the product buffer P through
 // the item tables; tasks with few open indices are made one product per thread.
 // A plan with any other task (or more operands than the kernel holds) keeps the
-// CUDA-core products.
+// CUDA-core products, and so does one that they serve faster (exact_pays).
 #include <algorithm>
+#include <cmath>
 #include <iterator>
 #include <map>
 #include <set>
@@ -210,6 +211,34 @@ void make_exact_split(const Plan& plan, ExactSplit* out) {
   ok &= S.wick_coefs.size() <= 65536;
   S.all = ok;
   *out = std::move(S);
+}
+
+// The estimates behind the choice, in us per slice on 152 SMs (one persistent CTA
+// each), fitted to the contraction stages of twelve lists (one channel to all 52 or
+// 90) on L = 8 .. 48 and met within 25%:
+//   digits: a launch, and per operand set as many rounds as it has products per SM,
+//     whose time has a constant part (the chunks of one product follow one another)
+//     and grows with the rows cut;
+//   CUDA cores: the chain of the longest task list, then the complex multiply-adds
+//     on the FP64 pipe or on the FP32 pipes (and a pass over the rows).
+// The digits read q-major blocks, whose forward transform takes 3 ps more per value
+// than the field-major one, but 5 ps less in double-float at L = 24 and 32 (two
+// passes, k_fft_xy_split).  Both sides measured, contraction in us:
+// double-float 48^3, channel 0: digits 5569, CUDA cores 3185 (the whole call 13958
+// and 11639); 52 channels: 13103 and 35969; 16^3, channel 0: 240 and 277; FP64 24^3,
+// channel 51: 710 and 608; channel 0: 712 and 1003; 8^3: 54 and 331.
+bool exact_pays(const Plan& plan, const ExactSplit& s, int L, bool df) {
+  const double V = (double)L * L * L, sms = 152;
+  double digits = 23 + V * plan.n_out * (df && (L == 24 || L == 32) ? -5e-6 : 3e-6);
+  for (int f = 0; f < kExactSets; f++) {
+    const ExactSet& x = s.set[f];
+    if (!x.nAp) continue;
+    if (f < kExactSlice) digits += std::ceil((V + 8) / 2 / sms) * (4 + 0.34 * x.nAp);
+    else digits += std::ceil(V / sms) * (2.5 + 0.027 * x.nAp + 0.0095 * x.nAp * (x.nBp - 16));
+  }
+  const double macs = (double)plan.pair_macs;
+  const double cores = df ? 130 + V * (0.018 + 1.83e-6 * macs) : 305 + V * 5.2e-6 * macs;
+  return digits < cores;
 }
 
 }  // namespace bbc

@@ -224,6 +224,8 @@ struct ExactSplit {
   std::vector<double> wick_coefs;                 // the distinct coefficients
 };
 void make_exact_split(const Plan& plan, ExactSplit* out);
+// whether the digit-sliced products of a whole split are faster than the CUDA-core ones
+bool exact_pays(const Plan& plan, const ExactSplit& s, int L, bool df);
 
 // Partition of the tasks into `groups` lists of near-equal cost (longest task
 // first to the cheapest list); each list is run by one warp for 32 q at a time.
