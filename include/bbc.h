@@ -376,8 +376,9 @@ bbc_status bbc_set_tuning(bbc_ctx* ctx, const bbc_tuning* t);
  * above, then (fused kernel) every valid (fused_warps, fused_steps,
  * fused_chunk) in row-major order (warps 8, 12, 16; steps 1, 2; chunks 0, 18,
  * 36, 72, 144) and then, with tensor cores, tc_kernel 0 and 1, or
- * (otherwise) pair_groups 48, 96, 192, 384 for the block-pair products --
- * keeps the fastest of each kernel, rebuilds slot 0 with
+ * (otherwise) pair_groups 48, 96, 192, 384 for the block-pair products (on the
+ * digit-sliced products, which have no lists, four timings of the same launch, and
+ * the value stays) -- keeps the fastest of each kernel, rebuilds slot 0 with
  * it, and records it for later contexts with the same L, precision and
  * channel list.  ms[i] (i < cap) receives the average milliseconds per launch
  * of candidate i (-1 for a candidate that is not valid here); *n_tried the

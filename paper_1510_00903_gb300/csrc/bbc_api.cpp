@@ -1129,10 +1129,13 @@ bbc_status bbc_autotune(bbc_ctx* c, int reps, bbc_tuning* best, double* ms, int 
       c->tune.tc_kernel = t.tc_kernel;
     }
   } else if (c->exact) {
-    // the digit-sliced products have no task lists: one timing stands for every pair_groups value
-    const double v = time_launches(c, reps, [&] { return launch_exact(c, 0); });
-    if (v < 0) return cuda_fail(c, cudaGetLastError(), "autotune: digit-sliced products");
-    for (size_t i = 0; i < sizeof(kPairGroupsCand) / sizeof(kPairGroupsCand[0]); i++) record(v);
+    // the digit-sliced products have no task lists: every pair_groups value is timed
+    // (they differ by noise only) and the context keeps its own
+    for (size_t i = 0; i < sizeof(kPairGroupsCand) / sizeof(kPairGroupsCand[0]); i++) {
+      const double v = time_launches(c, reps, [&] { return launch_exact(c, 0); });
+      record(v);
+      if (v < 0) return cuda_fail(c, cudaGetLastError(), "autotune: digit-sliced products");
+    }
   } else {  // block-pair products: task lists per 32 q
     const bool fp64 = fp64_storage(c->prec);
     const double* blks = c->d_blks;
