@@ -41,6 +41,9 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 #: 8 flops each: a complex product takes at least three real multiplications
 #: (Gauss), so at most 629 G FMA/s / 3 = 209.8 G complex MACs/s = 1.678 TFLOP/s
 FP64_CMAC_PEAK_TFLOPS = FP64_PEAK_TFLOPS * 8.0 / 6.0
+CMAC_PEAK_SOURCE = ("derived: 152 SM x 2 FP64 FMA/clk x 2070 MHz = 629.3 G FMA/s; a complex multiply-add (8 "
+                    "algorithmic flops) needs at least 3 real FMAs (three-multiplication complex product), so the "
+                    "FP64 pipe's ceiling is 209.8 G complex MACs/s = 1.678 TFLOP/s")
 #: FP32 FMA peak: 152 SMs x 128 lanes x 2 flop x 2070 MHz (probe: 74.8 TFLOP/s)
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
@@ -104,6 +107,27 @@ def profiled_traffic(path, kernel_src, pair_items):
     if fields.get("pair_items_per_q") != str(pair_items):
         return None
     return float(fields["dram_bytes_per_launch"])
+
+
+def exact_traffic(sizes, sites, df=False):
+    """DRAM bytes per launch of k_contract_exact from the committed summary of one 16^3 slice, for `sites` sites."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    name = "k_contract_exact_df_L16_slice.md" if df else "k_contract_exact_L16_slice.md"
+    t = profiled_traffic(os.path.join(here, "profiles", name),
+                         os.path.join(here, "paper_1510_00903_gb300", "csrc", "tc_exact.cu"), sizes["pair_items"])
+    return None if t is None else t * sites / L_BENCH ** 3
+
+
+def contraction_roofline(digits, achieved, df=False, traffic=None):
+    """Roofline entry of the FP64-accurate contraction: the digit-sliced products where the context has them
+    (``digits``), else the FP64 products on the CUDA cores."""
+    if not digits:
+        return {"bound": "alu", "kernel": "k_pair_products<double>", "achieved": achieved,
+                "peak": FP64_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_CMAC_PEAK_TFLOPS,
+                "traffic": None, "peak_source": CMAC_PEAK_SOURCE}
+    return {"bound": "tensor", "kernel": "k_contract_exact<dfr>" if df else "k_contract_exact<double>",
+            "achieved": achieved, "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": achieved / DIGIT_CMAC_PEAK_TFLOPS, "traffic": traffic, "peak_source": DIGIT_PEAK_SOURCE}
 
 
 #: diquark kind read by each sink-tensor family (the families' Gamma1 and the
@@ -450,10 +474,8 @@ def run_ours(args, torch, rank, world, local):
     c_avg_ms = c_ms / max(c_n, 1)
     flops_per_launch = 8.0 * sizes["pair_macs_per_site"] * V
     achieved = flops_per_launch / (c_avg_ms * 1e-3) / 1e12
-    roofline = {"bound": "tensor", "kernel": "k_contract_exact<double>", "achieved": achieved,
-                "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / DIGIT_CMAC_PEAK_TFLOPS,
-                "traffic": None, "peak_source": DIGIT_PEAK_SOURCE,
-                "algorithmic_flop_per_launch": flops_per_launch, "avg_launch_ms": c_avg_ms}
+    roofline = dict(contraction_roofline(True, achieved, traffic=exact_traffic(sizes, V)),
+                    algorithmic_flop_per_launch=flops_per_launch, avg_launch_ms=c_avg_ms)
     stage_ms = {k: v[0] / args.steps for k, v in stages.items()}
     step_roof = step_roofline(counts, V, T, stage_ms, ms, cmac_tflops=DIGIT_CMAC_PEAK_TFLOPS)
 
@@ -718,6 +740,7 @@ def run_decuplet(args, torch, dev, bbc, synth):
         if name == "fp64":
             clocks = sampler.summary()
         stages = bbc.bbc_stage_timing(cor.ctx)
+        digits = bbc.bbc_digit_products(cor.ctx)
         cor.close()
         ms = shard.max_over_ranks(e0.elapsed_time(e1) / args.steps, world, dev)
         c_ms, c_n = stages["contract"]
@@ -726,9 +749,12 @@ def run_decuplet(args, torch, dev, bbc, synth):
         legs[name] = {"value": shard.job_throughput(V * T * len(chans), world, ms), "ms_per_step": ms,
                       "stage_ms_per_step": stage_ms,
                       "contract_ms_per_slice": c_ms / max(c_n, 1),
-                      "contract_tflops": flop / (c_ms / max(c_n, 1) * 1e-3) / 1e12, "tuning": tune}
+                      "contract_tflops": flop / (c_ms / max(c_n, 1) * 1e-3) / 1e12, "digit_products": digits,
+                      "tuning": tune}
         if name != "df64":  # double-float arithmetic has no pipe peak of its own
-            legs[name]["step_roofline"] = step_roofline(counts, V, T, stage_ms, ms, mixed=name == "mixed")
+            legs[name]["step_roofline"] = step_roofline(
+                counts, V, T, stage_ms, ms, mixed=name == "mixed",
+                cmac_tflops=DIGIT_CMAC_PEAK_TFLOPS if digits else FP64_CMAC_PEAK_TFLOPS)
     if rank != 0:
         return
     fp = legs["fp64"]
@@ -739,10 +765,7 @@ def run_decuplet(args, torch, dev, bbc, synth):
                      "L": L, "T": T, "channels": len(chans),
                      "l2": f"no flush: block fields of one slice ({V * sizes['block_outputs'] * 16 / 1e6:.0f} MB) "
                            "exceed the 129 MB L2"},
-          "roofline": {"bound": "tensor", "kernel": "k_contract_exact<double>", "achieved": fp["contract_tflops"],
-                       "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s",
-                       "frac": fp["contract_tflops"] / DIGIT_CMAC_PEAK_TFLOPS, "traffic": None,
-                       "peak_source": DIGIT_PEAK_SOURCE},
+          "roofline": contraction_roofline(fp["digit_products"], fp["contract_tflops"]),
           "plan": sizes, "fp64": fp, "df64": legs["df64"], "mixed": legs["mixed"], "clocks": clocks})
 
 
@@ -997,7 +1020,7 @@ def run_default(args, torch, dev, bbc, synth):
             ach = 8.0 * sz["pair_macs_per_site"] * V2 / (ca * 1e-3) / 1e12
             leg["roofline"] = {"kernel": "k_contract_exact<double>", "achieved": round(ach, 4),
                                "peak": DIGIT_CMAC_PEAK_TFLOPS, "frac": round(ach / DIGIT_CMAC_PEAK_TFLOPS, 4),
-                               "traffic": None}
+                               "traffic": exact_traffic(sz, V2)}
         else:
             leg["err_vs_fp64"] = channel_errors(torch, out2[16], ref16)
         if prec in (bbc.BBC_FP64, bbc.BBC_MIXED_FP32):
@@ -1041,9 +1064,8 @@ def run_default(args, torch, dev, bbc, synth):
                 "h2d_bytes_per_step": int(HEAD_SLICES * 2 * V5 * 144 * 8),
                 "d2h_bytes_per_step": int(HEAD_SLICES * N_CH * V5 * 16 * 16)},
         "gpu_launches": launches,
-        "roofline": {"bound": "tensor", "kernel": "k_contract_exact<dfr>", "achieved": achieved,
-                     "peak": DIGIT_CMAC_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / DIGIT_CMAC_PEAK_TFLOPS,
-                     "traffic": None, "peak_source": DIGIT_PEAK_SOURCE, "avg_launch_ms": round(c_avg, 3)},
+        "roofline": dict(contraction_roofline(True, achieved, df=True, traffic=exact_traffic(sizes, V5, df=True)),
+                         avg_launch_ms=round(c_avg, 3)),
         "err_vs_fp64": head_err,
         "stage_ms_per_step": {k: round(v, 1) for k, v in stage_ms.items() if v > 0.5},
         # legs, one array each: [site*channels/s, ms per step, step roofline frac, max per-channel error vs FP64]
