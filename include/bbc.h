@@ -74,8 +74,8 @@ typedef enum {
 typedef enum {
   BBC_FP64 = 0,      /* blocks, FFTs, contraction and sums in FP64; the block-pair
                          products, where the plan allows, from 7-bit digits of 55-bit
-                         fixed-point values on the tensor cores: an error of about 2^-51
-                         of the product of the two rows' maxima.  A product below 2^-6 of
+                         fixed-point values on the tensor cores: an error of about 2^-52
+                         of the product of the two rows' bounds.  A product below 2^-6 of
                          that bound, or of a row with non-finite values or one below
                          2^-900, is made in FP64 instead, term by term */
   BBC_MIXED_FP32 = 1, /* blocks, FFTs and block-pair products in FP32 after an exact

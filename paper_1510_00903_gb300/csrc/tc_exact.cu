@@ -10,9 +10,9 @@
 // digit products of one weight ("level" s = i + j) of a complex product of
 // K = 144 terms add up to at most 8 x 288 x 64^2 < 2^24.  Levels 0 .. 7 are kept,
 // put together in 64-bit integers and rounded once.  The dropped levels leave an
-// error relative to the product of the two rows' maxima, not to the sum of the
-// terms' magnitudes: 7.5 units of 2^-54 of it rms for Gaussian rows, 16 (with a
-// mean of -15) for rows of one sign, 29 at the most in 10^5 emulated products.
+// error relative to the product of the two rows' bounds 2^e, not to the sum of the
+// terms' magnitudes: in units of 2^-54 of it 3.8 rms for Gaussian rows, 6.5 (with a
+// mean of -3.7) for rows of one sign, 24 at the most in 400,000 emulated products.
 // A product that comes out far below that bound, and any product of a row the
 // fixed point cannot hold, is therefore made again in the blocks' own arithmetic
 // (k_exact_wick).  (This is the splitting idea of Ozaki, Ogita, Oishi and
@@ -505,12 +505,13 @@ k_exact_small(const void* __restrict__ blk, int L, int n_out, const DevTask* __r
 //
 // Before the sums, products marked NaN are made again, a warp each, from the rows
 // in the blocks' own arithmetic: rows the digits do not hold, and products far
-// below the product of their rows' largest magnitudes.  The digits' error is about
-// 2^-51 of that bound (dropped levels and cut values): 2^-45 of a product at 2^-6 of
-// it, what bounds an FP64 sum of 288 terms; 2^-44, the operators' own error, at 2^-7
-// in double-float.  Where the large values of two rows meet (any field whose
+// below the product of their rows' bounds.  The digits' error is about 2^-52 of that,
+// at most 2^-49 seen (dropped levels and cut values): 2^-46 of a product at 2^-6 of
+// it, where 2^-45 bounds an FP64 sum of 288 terms, and 2^-45 at 2^-7 in double-float,
+// whose operators' own error is 2^-44.  Where the large values of two rows meet (any field whose
 // flavours are graded alike) under 0.1% of the products are made again; rows graded
-// against each other would lose theirs without it.  The marks and those products
+// against each other would lose theirs without it, and pay: with all products made
+// again the FP64 sums of 52 channels take 9.2 ms per 16^3 slice, the double-float ones 4.1.  The marks and those products
 // took the 16^3 sums of 52 channels from 121 to 150 us (FP64) and from 82 to 92
 // (double-float), and 48^3 ones from 1.65 to 1.96 ms.
 constexpr int kWickThreads = 256;

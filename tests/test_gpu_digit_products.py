@@ -143,3 +143,20 @@ def test_products_wait_self_test_needs_the_digit_products(bbc):
     assert bbc.bbc_check_products_wait(cor.ctx, 1) == bbc.BBC_ESTATE
     assert bbc.bbc_check_products_wait(cor.ctx, 0) == bbc.BBC_EINVAL
     cor.close()
+
+
+@pytest.mark.parametrize("precision,L,few,many", [(0, 24, [51], range(10, 52)), (0, 24, [64], range(64, 154)),
+                                                  (3, 16, [14], range(10, 52)), (3, 24, [64], range(64, 154)),
+                                                  (3, 32, [0, 51], range(52)), (3, 48, [51], range(10, 52))])
+def test_few_channels_on_the_cuda_cores_agree_with_the_digits(bbc, precision, L, few, many):
+    """The same channels from a list short enough for the CUDA cores and from one on the digit products."""
+    gen = torch.Generator(device="cuda").manual_seed(13 + L)
+    Sl, Ss = (_normal(gen, (L ** 3, 12, 12)) for _ in range(2))
+    many, routes = list(many), []
+    for chans in (few, many):
+        ctx = bbc.bbc_create(L, 4, 0, 0.3, 0.4, precision, chans)
+        routes.append(bbc.bbc_digit_products(ctx))
+        bbc.bbc_destroy(ctx)
+    assert routes == [False, True]
+    got, want = _run(bbc, L, Sl, Ss, few, precision), _run(bbc, L, Sl, Ss, many, precision)
+    assert _err(got, want[[many.index(c) for c in few]]) <= TOL
