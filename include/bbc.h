@@ -75,7 +75,7 @@ typedef enum {
   BBC_FP64 = 0,      /* blocks, FFTs, contraction and sums in FP64; the block-pair
                          products, where the plan allows, from 7-bit digits of 55-bit
                          fixed-point values on the tensor cores: an error of about 2^-52
-                         of the product of the two rows' bounds.  A product below 2^-6 of
+                         of the product of the two rows' bounds.  A product below 2^-7 of
                          that bound, or of a row with non-finite values or one below
                          2^-900, is made in FP64 instead, term by term */
   BBC_MIXED_FP32 = 1, /* blocks, FFTs and block-pair products in FP32 after an exact
@@ -103,7 +103,7 @@ typedef enum {
                          (unevaluated sums of two FP32 values, 48-bit significand) on
                          the FP32 pipes: propagators, blocks, FFTs and Wick sums; the
                          block-pair products as for BBC_FP64 (in double-float
-                         where below 2^-7 of the bound, or of a row below 2^-72); FP64
+                         where made term by term, and for rows below 2^-72); FP64
                          only to split the input and to normalise */
   BBC_MIXED_TF32 = 4  /* trial: as BBC_MIXED_FP32, with the tensor-core operands rounded
                          once to TF32 (10-bit mantissa, round to nearest) instead of

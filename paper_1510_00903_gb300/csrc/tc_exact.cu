@@ -80,14 +80,15 @@ constexpr int kXFixed = 2048;                  // static shared memory (at most)
 constexpr int kXBad = 0x7000, kXZero = -0x3000, kXNone = 0x2000;
 // Per block type: rows and products below 2^kLow and 2^kLowProduct (the digits of
 // an FP64 value are cut by at most 63 bits, double-float scales are FP32 numbers; a
-// product keeps a normal result), and a product below 2^-kFar of the rows'
+// product keeps a normal result), and a product below 2^-kXFar of the rows'
 // bound is not trusted (k_exact_wick).
 template <typename T>
 struct XLimits;
 template <>
-struct XLimits<double> { static constexpr int kLow = -900, kLowProduct = -900, kFar = 6; };
+struct XLimits<double> { static constexpr int kLow = -900, kLowProduct = -900; };
 template <>
-struct XLimits<dfr> { static constexpr int kLow = -72, kLowProduct = -90, kFar = 7; };
+struct XLimits<dfr> { static constexpr int kLow = -72, kLowProduct = -90; };
+constexpr int kXFar = 7;
 
 __device__ __forceinline__ uint32_t x_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -504,16 +505,18 @@ k_exact_small(const void* __restrict__ blk, int L, int n_out, const DevTask* __r
 // every 16 terms.
 //
 // Before the sums, products marked NaN are made again, a warp each, from the rows
-// in the blocks' own arithmetic: rows the digits do not hold, and products far
-// below the product of their rows' bounds.  The digits' error is about 2^-52 of that,
-// at most 2^-49 seen (dropped levels and cut values): 2^-46 of a product at 2^-6 of
-// it, where 2^-45 bounds an FP64 sum of 288 terms, and 2^-45 at 2^-7 in double-float,
-// whose operators' own error is 2^-44.  Where the large values of two rows meet (any field whose
-// flavours are graded alike) under 0.1% of the products are made again; rows graded
-// against each other would lose theirs without it, and pay: with all products made
-// again the FP64 sums of 52 channels take 9.2 ms per 16^3 slice, the double-float ones 4.1.  The marks and those products
-// took the 16^3 sums of 52 channels from 121 to 150 us (FP64) and from 82 to 92
-// (double-float), and 48^3 ones from 1.65 to 1.96 ms.
+// in the blocks' own arithmetic: rows the digits do not hold, and products below
+// 2^-kXFar of the product of their rows' bounds.  The digits' error is about 2^-52 of
+// that, at most 2^-49 seen (dropped levels and cut values), so about 2^-45 of a product
+// at 2^-7 of it: what bounds an FP64 sum of 288 terms, and half the double-float
+// operators' own error.  Where the large values of two rows meet (any field whose
+// flavours are graded alike) under 0.03% of the products are made again, mostly at
+// q = 0 of smooth fields; at 2^-6 four times as many, and the CTA of that q held up
+// small lattices (Lambda N 8^3, FP64: 22 against 16 us per slice).  Rows graded against
+// each other would lose their products without it, and pay: with all of them made again
+// the sums of 52 channels take 9.2 ms per 16^3 slice in FP64, 4.1 in double-float.
+// The marks and those products took the 16^3 sums of 52 channels from 121 to 142 us
+// (FP64) and from 82 to 92 (double-float), and 48^3 ones from 1.65 to 1.97 ms.
 constexpr int kWickThreads = 256;
 struct WickAcc64 {
   double x = 0, y = 0;
@@ -988,7 +991,7 @@ __device__ __forceinline__ void exact_set(unsigned char* smem, XShared& xs, cons
         // the sum is (sum of T_A T_B) 2^-56, T = x 2^(55 - e): 2^54 stands for the
         // product of the rows' bounds.  NaN marks what k_exact_wick makes again.
         const int e = s_ex[row] + s_ey[col], hr = (int)(re >> 32), hi = (int)(im >> 32);
-        const bool far = max(hr ^ (hr >> 31), hi ^ (hi >> 31)) < (1 << (22 - XLimits<T>::kFar));
+        const bool far = max(hr ^ (hr >> 31), hi ^ (hi >> 31)) < (1 << (22 - kXFar));
         const bool again = e > kXNone || (e >= -kXNone && (far || e < XLimits<T>::kLowProduct));
         const Ld v = x_value(Ld(), re, im, again ? kXBad : e - 54);
         const int item_q = (int)(short)en.y, item_n = en.y >> 16;
